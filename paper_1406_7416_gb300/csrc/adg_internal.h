@@ -299,6 +299,30 @@ __device__ __forceinline__ void euler_fluxes(const T* Q, T gm1, T (*F)[D + 2]) {
   }
 }
 
+// euler_fluxes in FP64 with the off-diagonal momentum products m_j v_k = m_k v_j
+// formed once (16 FP64 operations and the division in 2D, 22 in 3D).
+template <int D>
+__device__ __forceinline__ void euler_fluxes_sym(const double* Q, double gm1, double (*F)[D + 2]) {
+  const double r = 1.0 / Q[0];
+  double v[D];
+  double kin = 0.0;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    v[k] = Q[1 + k] * r;
+    kin += Q[1 + k] * v[k];
+  }
+  const double p = gm1 * (Q[D + 1] - 0.5 * kin);
+  const double Ep = Q[D + 1] + p;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    F[k][0] = Q[1 + k];
+    F[k][1 + k] = Q[1 + k] * v[k] + p;
+#pragma unroll
+    for (int j = k + 1; j < D; ++j) F[k][1 + j] = F[j][1 + k] = Q[1 + j] * v[k];
+    F[k][D + 1] = v[k] * Ep;
+  }
+}
+
 // Conversions and tests on the integer pipe.  GB300 runs every FP64
 // instruction -- conversions between FP32 and FP64 and FP64 comparisons
 // included -- on its narrow FP64 pipe (about the rate of an FP64 FMA, measured),

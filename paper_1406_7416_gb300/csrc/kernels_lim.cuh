@@ -6,6 +6,7 @@
 // troubled-cell list, in chunks of `chunk` cells that share the scratch.
 #pragma once
 
+#include "fixed.cuh"
 #include "kernels_dg.cuh"
 
 namespace adg {
@@ -434,8 +435,7 @@ __global__ void __launch_bounds__(256) k_lim_sweep(Batch bt, int pass) {
 // L4: degree-2 space-time predictor (Eq. pde.nc.dg2 with 3 GL nodes per axis
 // and in time, 3 Picard sweeps) on the subcells whose traces the sub-face
 // fluxes use: the Ns^d interior subcells and the Ns^(d-1) ghost subcells
-// facing each of the 2d cell faces.  In mixed precision the first two sweeps
-// run in FP32 and the last in FP64.
+// facing each of the 2d cell faces.
 constexpr int SUBS_PER_BLOCK_2D = 4;
 constexpr int SUBS_PER_BLOCK_3D = 2;
 
@@ -470,24 +470,22 @@ __device__ __forceinline__ int cross_subcell(int r) {
   return c[0] + NE * (c[1] + NE * c[2]);
 }
 
-// n32: sweeps (of 3) run in FP32 before the FP64 ones (MIXED only; the same
-// for the whole launch, so every block takes the same barriers).
-// QF: the whole predictor in FP32 (n32 = 3) from an FP32 reconstruction, the
-// space-time nodal values stored in FP32 (qsub read as float by k_lim_flux).
-template <int D, int N, bool MIXED, typename WT, bool QF>
+// L4 in mixed precision with some sweeps in each precision: n32 (1..3) of the
+// three run in FP32, the others in FP64 after them (the same n32 for the whole
+// launch, so every block takes the same barriers).  WT: the element type of
+// the reconstruction.
+template <int D, int N, typename WT>
 __global__ void __launch_bounds__(256) k_lim_predict(Batch bt, int pass, int n32) {
   using DM = Dims<D, N>;
   constexpr int NV = DM::NV, NST3 = DM::NST3, ND3 = DM::ND3, NED = DM::NED, Ns = DM::Ns;
   constexpr int NCROSS = DM::NSD + 2 * D * DM::NSF;
   constexpr int SPB = (D == 2) ? SUBS_PER_BLOCK_2D : SUBS_PER_BLOCK_3D;
-  constexpr int SPBF = MIXED ? SPB : 1;
-  constexpr int SPBD = QF ? 1 : SPB;           // FP64 staging (unused when QF)
-  __shared__ double su[SPBD][NV * ND3];
-  __shared__ double sq[SPBD][NV * NST3];
-  __shared__ double sF[SPBD][D * NV * NST3];
-  __shared__ float suf[SPBF][NV * ND3];
-  __shared__ float sqf[SPBF][NV * NST3];
-  __shared__ float sFf[SPBF][D * NV * NST3];
+  __shared__ double su[SPB][NV * ND3];
+  __shared__ double sq[SPB][NV * NST3];
+  __shared__ double sF[SPB][D * NV * NST3];
+  __shared__ float suf[SPB][NV * ND3];
+  __shared__ float sqf[SPB][NV * NST3];
+  __shared__ float sFf[SPB][D * NV * NST3];
   __shared__ double D3[9], K3[9];
   __shared__ float D3f[9], K3f[9];
   if (threadIdx.x < 9) {
@@ -521,33 +519,6 @@ __global__ void __launch_bounds__(256) k_lim_predict(Batch bt, int pass, int n32
     const double gm1 = p.gamma - 1.0;
     const WT* W = reinterpret_cast<const WT*>(p.b.sweep[D - 1]);   // [j][v][NED][ND3]
     __syncthreads();
-    if constexpr (QF) {
-      if (live)
-        for (int e = lt; e < NV * ND3; e += NST3) {
-          const int v = e / ND3, i = e - v * ND3;
-          suf[grp][e] = (float)W[((j * NV + v) * NED + sc) * ND3 + i];
-        }
-      __syncthreads();
-      if (live)
-        for (int e = lt; e < NV * NST3; e += NST3) {
-          const int v = e / NST3, l = e - v * NST3;
-          sqf[grp][e] = suf[grp][v * ND3 + (l % ND3)];
-        }
-      __syncthreads();
-      for (int it = 0; it < 3; ++it) {
-        if (live) picard_flux<D, 3, float>(sqf[grp], sFf[grp], (float)gm1, lt, NST3);
-        __syncthreads();
-        if (live) picard_deriv_sub<D>(sFf[grp], sqf[grp], cf, lt, NST3);
-        __syncthreads();
-        if (live) picard_time_sub<D>(sqf[grp], suf[grp], lt, NST3);
-        __syncthreads();
-      }
-      if (live) {
-        float* dst = reinterpret_cast<float*>(p.b.qsub) + ((size_t)j * NED + sc) * (size_t)(NV * NST3);
-        for (int e = lt; e < NV * NST3; e += NST3) dst[e] = sqf[grp][e];
-      }
-      continue;
-    }
     if (live) {
       for (int e = lt; e < NV * ND3; e += NST3) {
         const int v = e / ND3, i = e - v * ND3;
@@ -555,35 +526,26 @@ __global__ void __launch_bounds__(256) k_lim_predict(Batch bt, int pass, int n32
       }
     }
     __syncthreads();
-    int it0 = 0;
-    if (MIXED && n32 > 0) {
-      if (live) {
-        for (int e = lt; e < NV * ND3; e += NST3) suf[grp][e] = (float)su[grp][e];
-        for (int e = lt; e < NV * NST3; e += NST3) {
-          const int v = e / NST3, l = e - v * NST3;
-          sqf[grp][e] = (float)su[grp][v * ND3 + (l % ND3)];
-        }
-      }
-      __syncthreads();
-      for (int it = 0; it < n32; ++it) {
-        if (live) picard_flux<D, 3, float>(sqf[grp], sFf[grp], (float)gm1, lt, NST3);
-        __syncthreads();
-        if (live) picard_deriv<D, 3, float>(sFf[grp], sqf[grp], D3f, cf, lt, NST3);
-        __syncthreads();
-        if (live) picard_time<D, 3, float>(sqf[grp], suf[grp], K3f, lt, NST3);
-        __syncthreads();
-      }
-      if (live)
-        for (int e = lt; e < NV * NST3; e += NST3) sq[grp][e] = (double)sqf[grp][e];
-      it0 = n32;
-    } else if (live) {
+    if (live) {
+      for (int e = lt; e < NV * ND3; e += NST3) suf[grp][e] = (float)su[grp][e];
       for (int e = lt; e < NV * NST3; e += NST3) {
         const int v = e / NST3, l = e - v * NST3;
-        sq[grp][e] = su[grp][v * ND3 + (l % ND3)];
+        sqf[grp][e] = (float)su[grp][v * ND3 + (l % ND3)];
       }
     }
     __syncthreads();
-    for (int it = it0; it < 3; ++it) {
+    for (int it = 0; it < n32; ++it) {
+      if (live) picard_flux<D, 3, float>(sqf[grp], sFf[grp], (float)gm1, lt, NST3);
+      __syncthreads();
+      if (live) picard_deriv<D, 3, float>(sFf[grp], sqf[grp], D3f, cf, lt, NST3);
+      __syncthreads();
+      if (live) picard_time<D, 3, float>(sqf[grp], suf[grp], K3f, lt, NST3);
+      __syncthreads();
+    }
+    if (live)
+      for (int e = lt; e < NV * NST3; e += NST3) sq[grp][e] = (double)sqf[grp][e];
+    __syncthreads();
+    for (int it = n32; it < 3; ++it) {
       if (live) picard_flux<D, 3, double>(sq[grp], sF[grp], gm1, lt, NST3);
       __syncthreads();
       if (live) picard_deriv<D, 3, double>(sF[grp], sq[grp], D3, c, lt, NST3);
@@ -598,11 +560,198 @@ __global__ void __launch_bounds__(256) k_lim_predict(Batch bt, int pass, int n32
   }
 }
 
+// L4 in FP64: the subcell predictor in registers with its contractions on the
+// integer pipes (fixed.cuh).  What bounds the FP64 limiter is the FP64 pipe (two
+// operations per clock and multiprocessor): of the 22 FP64 operations that a
+// 3D space-time node and variable cost per sweep, 16 were the contractions.
+//
+// Lane l works on spatial node l (3D: 27 nodes of one subcell; 2D: 9 nodes of
+// each of three subcells) and holds its three time nodes.  The fluxes F_k of a
+// time node are put on one scale per subcell and variable (the largest
+// magnitude over its nodes and axes; a smooth subcell's values lie within the
+// 6 bits that scale keeps below FP64's), the three operands of each line come
+// from the lanes on it as integers by shuffles, and S = sum_k (c_k D) x_k F_k
+// is one exact integer sum over the axes: c_k is folded into the operator once
+// per state.  The time solve acts on the lane's own S, brought to the largest
+// of its three scales, and only its result becomes a double again:
+// q = u - Ktau S.  The first sweep starts from u (x) 1: one space term, and
+// q_m = u - kappa_m S with kappa = Ktau 1.  FP64 operations per sweep, node and
+// variable: the flux (4.4 in 3D, 4.1 in 2D) and one subtraction.
+//
+// Measured (GB300, 3D explosion 33 x 29 x 30, N = 3): 56 ms for 5611 troubled
+// cells (3.6 million subcells; FP64 pipe 72% busy, 208 FP64 instructions per
+// subcell), the former kernel with FP64 contractions from shared memory 174 ms
+// for 4883 (mean of two launches); 2D N = 5, 146 patches: 351 -> 100 us.
+template <int D, int N, typename WT>
+__global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
+  using DM = Dims<D, N>;
+  constexpr int NV = DM::NV, NST3 = DM::NST3, ND3 = DM::ND3, NED = DM::NED, Ns = DM::Ns;
+  constexpr int NCROSS = DM::NSD + 2 * D * DM::NSF;
+  constexpr int SPW = D == 2 ? 3 : 1;                   // subcells per warp
+  constexpr unsigned FULL = 0xffffffffu;
+  __shared__ FxOp K3[9], kap[3];                        // Ktau and its row sums
+  __shared__ int s_gK;
+  const Ops* o = bt.pps[0]->ops;                        // (the subcell operators do not depend on N)
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 32) {
+    // scale exponents from the row sums, then one entry per lane
+    double ks = 0.0;
+    for (int m = 0; m < 3; ++m) {
+      const double r = fabs(o->Kt3[3 * m]) + fabs(o->Kt3[3 * m + 1]) + fabs(o->Kt3[3 * m + 2]);
+      ks = r > ks ? r : ks;
+    }
+    const int gK = fx_scale(ks);
+    if (lane < 9) K3[lane] = fx_op(o->Kt3[lane], gK);
+    else if (lane < 12) {
+      const double* r = o->Kt3 + 3 * (lane - 9);
+      kap[lane - 9] = fx_op(r[0] + r[1] + r[2], gK);
+    }
+    if (lane == 0) s_gK = gK;
+  }
+  __syncthreads();
+  const int gK = s_gK;
+  const int l = lane < 27 ? lane : 26;                  // idle lanes mirror lane 26
+  const int grp = D == 2 ? l / 9 : 0, node = l - grp * ND3;
+  const int a = node % 3, b = (node / 3) % 3, c = D == 3 ? node / 9 : 0;
+  const int sx = l - a, sy = l - 3 * b, sz = l - 9 * c; // first lanes of this node's lines
+  FxOp row[D][3] = {};                                  // this node's rows of c_k D3
+  int gD = 0, state = -1;
+  const int wpb = blockDim.x >> 5;
+  const long long total = bt.pre[bt.n] * NCROSS;
+  const long long groups = (total + SPW - 1) / SPW;
+  for (long long gi = (long long)blockIdx.x * wpb + (threadIdx.x >> 5); gi < groups;
+       gi += (long long)gridDim.x * wpb) {
+    const long long item = gi * SPW + grp;
+    const bool live = item < total && lane < 27;
+    const long long tg = item < total ? item / NCROSS : bt.pre[bt.n] - 1;
+    const LimItem it = lim_item(bt, tg);
+    const Params& p = *bt.pps[it.s];
+    const long long j0 = it.j;
+    const int sc = item < total ? cross_subcell<D, Ns>((int)(item - tg * NCROSS)) : cross_subcell<D, Ns>(0);
+    if (__any_sync(FULL, it.s != state)) {
+      // the rows of c_k D3 of this lane's state (they change with its step)
+      state = it.s;
+      double cs = 0.0, rs = 0.0;
+#pragma unroll
+      for (int k = 0; k < D; ++k) cs += p.b.coef[3 + k];
+      for (int m = 0; m < 3; ++m) {
+        const double r = fabs(o->D3[3 * m]) + fabs(o->D3[3 * m + 1]) + fabs(o->D3[3 * m + 2]);
+        rs = r > rs ? r : rs;
+      }
+      gD = fx_scale(cs * rs);
+#pragma unroll
+      for (int k = 0; k < D; ++k) {
+        const int ak = k == 0 ? a : (k == 1 ? b : c);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) row[k][j] = fx_op(p.b.coef[3 + k] * o->D3[ak * 3 + j], gD);
+      }
+    }
+    const double gm1 = p.gamma - 1.0;
+    const WT* W = reinterpret_cast<const WT*>(p.b.sweep[D - 1]);   // [j][v][NED][ND3]
+    double u[NV], q[3][NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) u[v] = (double)W[((j0 * NV + v) * NED + sc) * ND3 + node];
+    // S = sum_k c_k D x_k F_k(Q) at this node: Sv[v] 2^64 on the scale es[v]
+    auto space_term = [&](const double* Q, long long* Sv, unsigned* es) {
+      double F[D][D + 2];
+      euler_fluxes_sym<D>(Q, gm1, F);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        unsigned key = fx_key(F[0][v]);
+#pragma unroll
+        for (int k = 1; k < D; ++k) key = max(key, fx_key(F[k][v]));
+        unsigned e;
+        if constexpr (D == 3) {
+          e = __reduce_max_sync(FULL, key) >> 21;
+        } else {
+          const unsigned e0 = __reduce_max_sync(FULL, grp == 0 ? key : 0u);
+          const unsigned e1 = __reduce_max_sync(FULL, grp == 1 ? key : 0u);
+          const unsigned e2 = __reduce_max_sync(FULL, grp == 2 ? key : 0u);
+          e = (grp == 0 ? e0 : (grp == 1 ? e1 : e2)) >> 21;
+        }
+        const unsigned ec = max(e, FX_E_MIN);
+        FxAcc acc;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+          const int base = k == 0 ? sx : (k == 1 ? sy : sz);
+          const int st = k == 0 ? 1 : (k == 1 ? 3 : 9);
+          const FxVal f = fx_val(F[k][v], ec);
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            FxVal x;
+            x.h = __shfl_sync(FULL, f.h, base + j * st);
+            x.l = __shfl_sync(FULL, f.l, base + j * st);
+            acc.add(x, row[k][j]);
+          }
+        }
+        Sv[v] = e < FX_E_MIN ? 0 : acc.sum();
+        es[v] = e;
+      }
+    };
+    // u - (R as a double), R on the scale of a dot product of S by Ktau
+    auto close = [&](double u0, long long R, unsigned e) {
+      const int bf = (int)e + gD + gK + 6;
+      double x = fx_double(R, bf);
+      if (bf < 70) x = 0.0;
+      if (e >= FX_E_MAX || bf > 2040) x = __longlong_as_double(0x7ff8000000000000LL);
+      return u0 - x;
+    };
+    {
+      long long S[NV];
+      unsigned es[NV];
+      space_term(u, S, es);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        FxVal x;
+        x.l = (int)S[v];
+        x.h = (int)((S[v] - x.l) >> 32);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          FxAcc acc;
+          acc.add(x, kap[m]);
+          q[m][v] = close(u[v], acc.sum(), max(es[v], FX_E_MIN));
+        }
+      }
+    }
+#pragma unroll 1
+    for (int sweep = 1; sweep < 3; ++sweep) {
+      long long S[3][NV];
+      unsigned es[3][NV];
+#pragma unroll
+      for (int m = 0; m < 3; ++m) space_term(q[m], S[m], es[m]);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const unsigned e = max(max(es[0][v], es[1][v]), max(es[2][v], FX_E_MIN));
+        FxVal x[3];
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          const unsigned sh = e - max(es[m][v], FX_E_MIN);
+          const long long s = S[m][v] >> (sh < 63u ? sh : 63u);
+          x[m].l = (int)s;
+          x[m].h = (int)((s - x[m].l) >> 32);
+        }
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          FxAcc acc;
+#pragma unroll
+          for (int j = 0; j < 3; ++j) acc.add(x[j], K3[m * 3 + j]);
+          q[m][v] = close(u[v], acc.sum(), e);
+        }
+      }
+    }
+    if (live) {
+      double* dst = p.b.qsub + ((size_t)j0 * NED + sc) * (size_t)(NV * NST3);
+#pragma unroll
+      for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int m = 0; m < 3; ++m) dst[v * NST3 + m * ND3 + node] = q[m][v];
+    }
+  }
+}
+
 // L4 in mixed precision with the whole subcell predictor in FP32 (the default
 // of the FP32 subcell scheme): one warp per subcell, W subcells per block,
-// each warp synchronised by __syncwarp alone (the per-subcell arithmetic of
-// k_lim_predict's QF path, none of its block barriers, and no thread group
-// straddling two warps).  The blocks loop over the pass's subcells.
+// each warp synchronised by __syncwarp alone.  The blocks loop over the pass's subcells.
 template <int D>
 struct LimWarps {
   static constexpr int W = (D == 2) ? 8 : 4;     // subcells per block (static shared memory)

@@ -205,6 +205,15 @@ struct Launch {
     return cudaGetLastError();
   }
 
+  // The FP64 subcell predictor on `ncross` subcells at most, persistent.
+  template <typename WT>
+  static void launch_predict_i(const Batch& lim, long long ncross, cudaStream_t s) {
+    constexpr int SPW = D == 2 ? 3 : 1;
+    static const int gw = persistent_grid(k_lim_predict_i<D, N, WT>, 128, 0, 1LL << 40);
+    const long long want = ((ncross + SPW - 1) / SPW + 3) / 4;
+    k_lim_predict_i<D, N, WT><<<(int)(want < gw ? want : gw), 128, 0, s>>>(lim);
+  }
+
   // One limiter pass (pass < 0: the pass of the device-sized loop).
   static cudaError_t lim_pass(const StepLaunch& sl, int pass, cudaStream_t s) {
     cudaError_t e;
@@ -256,16 +265,18 @@ struct Launch {
           const long long want = (ncross + W - 1) / W;
           k_lim_predict_w<D, N><<<(int)(want < gw ? want : gw), 32 * W, 0, s>>>(lim);
         }
-      } else
-        k_lim_predict<D, N, true, float, false><<<gp, SPB * DM::NST3, 0, s>>>(lim, pass, sl.sub32);
+      } else if (sl.sub32 > 0)
+        k_lim_predict<D, N, float><<<gp, SPB * DM::NST3, 0, s>>>(lim, pass, sl.sub32);
+      else
+        launch_predict_i<float>(lim, ncross, s);
     } else {
       k_lim_sweep<D, N, 0, double><<<gs, 256, 0, s>>>(lim, pass);
       k_lim_sweep<D, N, 1, double><<<gs, 256, 0, s>>>(lim, pass);
       if (D == 3) k_lim_sweep<D, N, (D == 3 ? 2 : 1), double><<<gs, 256, 0, s>>>(lim, pass);
-      if (sl.prec == ADG_PREC_MIXED_FP32)
-        k_lim_predict<D, N, true, double, false><<<gp, SPB * DM::NST3, 0, s>>>(lim, pass, sl.sub32);
+      if (sl.prec == ADG_PREC_MIXED_FP32 && sl.sub32 > 0)
+        k_lim_predict<D, N, double><<<gp, SPB * DM::NST3, 0, s>>>(lim, pass, sl.sub32);
       else
-        k_lim_predict<D, N, false, double, false><<<gp, SPB * DM::NST3, 0, s>>>(lim, pass, 0);
+        launch_predict_i<double>(lim, ncross, s);
     }
     const int gf = grid_for(ch * (Ns + 1) * DM::NSF, 256);
     if (traces && D == 2) {

@@ -152,7 +152,6 @@ struct NoAlloc {
                          double dt, double* vnew, double* faces, cudaStream_t s) {
     k_noalloc_begin<<<1, 32, 0, s>>>(p.b.counters, p.b.dt, pps, pre, pdev, count, dt);
     if (count == 0) return cudaGetLastError();
-    constexpr int SPB = (D == 2) ? SUBS_PER_BLOCK_2D : SUBS_PER_BLOCK_3D;
     const long long ch = count;
     const Batch lim{pps, 1, pre};
     k_lim_sweep<D, N, 0, double><<<grid_for(ch * DM::NV * DM::LD, 256), 256, 0, s>>>(lim, 0);
@@ -160,7 +159,7 @@ struct NoAlloc {
     if (D == 3)
       k_lim_sweep<D, N, (D == 3 ? 2 : 1), double><<<grid_for(ch * DM::NV * DM::LD, 256), 256, 0, s>>>(lim, 0);
     const long long ncross = ch * (DM::NSD + 2 * D * DM::NSF);
-    k_lim_predict<D, N, false, double, false><<<grid_for(ncross, SPB, kNumSM * 16), SPB * DM::NST3, 0, s>>>(lim, 0, 0);
+    Launch<D, N>::template launch_predict_i<double>(lim, ncross, s);
     k_lim_flux<D, N, 0, double, double><<<grid_for(ch * (DM::Ns + 1) * DM::NSF, 256), 256, 0, s>>>(lim, 0);
     k_lim_flux<D, N, 1, double, double><<<grid_for(ch * (DM::Ns + 1) * DM::NSF, 256), 256, 0, s>>>(lim, 0);
     if (D == 3)
