@@ -307,43 +307,63 @@ __global__ void __launch_bounds__(128) k_lim_patch(Batch bt, int pass) {
 
 
 // 1D WENO3 on five consecutive subcell averages u[0..4] (target subcell u[2]):
-// values of the reconstruction at the 3 GL nodes of the target subcell.
-// Weights w_k = lambda_k / t_k, t_k = (sigma_k + eps)^8, normalised; with
-// a_k = lambda_k prod_{j != k} t_j the normalised weights are a_k / sum a, so
-// one division serves all outputs (the plain form is used if a product of
-// two t_j could overflow).
+// values of the reconstruction at the 3 GL nodes x = 1/2, 1/2 -+ y of the
+// target subcell, y^2 = 3/20.
+//
+// The FP64 pipe bounds the sweeps, so the stencils are written in the first
+// and second differences they share.  The parabola of stencil k has the average
+// u[2] over the target, the slope b_k at its middle and the second derivative
+// s_k (the stencil's second difference):
+//   p_k(x) = u[2] + b_k (x - 1/2) + s_k ((x - 1/2)^2 / 2 - 1/24),
+//   sigma_k = int_0^1 (p')^2 + (p'')^2 = b_k^2 + 13/12 s_k^2,
+// and the interface slopes d1 = u[2] - u[1], d2 = u[3] - u[2] give
+//   b = d1 + s_0 / 2, d1 + s_1 / 2, d2 - s_2 / 2.
+// About 54 FP64 operations, the division among them; in the monomials of each
+// stencil they were about 97.
+//
+// Weights w_k = lambda_k / (sigma_k + eps)^8, normalised: with t_k the
+// sigma_k + eps over the power of two of the smallest and a_k = lambda_k
+// prod_{j != k} t_j^8 they are a_k / sum a, one division.  t_k is cut at 2^50,
+// where the stencil's weight is below 2^-380 of the largest, so that no
+// product overflows whatever the data's magnitude.
+//
+// Measured (GB300, 3D explosion 33 x 29 x 30, N = 3): the three sweeps of 5611
+// troubled cells 30.2 ms; in the monomial form 46.1 ms for 4883 (means of two
+// launches).  2D N = 5, 146 patches: 94 -> 60 us.
+__device__ __forceinline__ double weno_scaled(double t, int emin) {
+  // (exponent field and mantissa of a positive number, by integer operations)
+  int hi = __double2hiint(t) - emin;
+  const int cut = (1023 + 50) << 20;
+  const bool far = hi >= cut;
+  return far ? __hiloint2double(cut, 0) : __hiloint2double(hi, __double2loint(t));
+}
+
 __device__ __forceinline__ void weno3(const double* u, const Ops* __restrict__ o, double* out) {
-  double t[3], p0[3], p1[3], p2[3];
+  const double d0 = u[1] - u[0], d1 = u[2] - u[1], d2 = u[3] - u[2], d3 = u[4] - u[3];
+  const double s[3] = {d1 - d0, d2 - d1, d3 - d2};
+  const double b[3] = {fma(0.5, s[0], d1), fma(0.5, s[1], d1), fma(-0.5, s[2], d2)};
+  double t[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) t[k] = fma(b[k], b[k], fma((13.0 / 12.0) * s[k], s[k], WENO_EPS));
+  // over the smallest's power of two (t >= eps > 0; NaN stays in b and s)
+  const int h0 = __double2hiint(t[0]), h1 = __double2hiint(t[1]), h2 = __double2hiint(t[2]);
+  const int emin = (min(h0, min(h1, h2)) & 0x7ff00000) - (1023 << 20);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const double* C = o->C[k];
-    const double c0 = C[0] * u[k] + C[1] * u[k + 1] + C[2] * u[k + 2];
-    const double c1 = C[3] * u[k] + C[4] * u[k + 1] + C[5] * u[k + 2];
-    const double c2 = C[6] * u[k] + C[7] * u[k + 1] + C[8] * u[k + 2];
-    // sigma = int_0^1 (p')^2 + (p'')^2 = c1^2 + 2 c1 c2 + 16/3 c2^2
-    const double sigma = c1 * (c1 + 2.0 * c2) + (16.0 / 3.0) * c2 * c2;
-    double tk = sigma + WENO_EPS;
-    tk = tk * tk;
-    tk = tk * tk;
-    t[k] = tk * tk;
-    p0[k] = c0 + c1 * o->E[1] + c2 * o->E[2];
-    p1[k] = c0 + c1 * o->E[4] + c2 * o->E[5];
-    p2[k] = c0 + c1 * o->E[7] + c2 * o->E[8];
+    double x = weno_scaled(t[k], emin);
+    x = x * x;
+    x = x * x;
+    t[k] = x * x;
   }
-  double a0, a1, a2;
-  if (t[0] < 1e150 && t[1] < 1e150 && t[2] < 1e150) {
-    a0 = t[1] * t[2];
-    a1 = WENO_LAMBDA_C * (t[0] * t[2]);
-    a2 = t[0] * t[1];
-  } else {
-    a0 = 1.0 / t[0];
-    a1 = WENO_LAMBDA_C / t[1];
-    a2 = 1.0 / t[2];
-  }
+  const double a0 = t[1] * t[2], a1 = WENO_LAMBDA_C * (t[0] * t[2]), a2 = t[0] * t[1];
   const double inv = 1.0 / (a0 + a1 + a2);
-  out[0] = (a0 * p0[0] + a1 * p0[1] + a2 * p0[2]) * inv;
-  out[1] = (a0 * p1[0] + a1 * p1[1] + a2 * p1[2]) * inv;
-  out[2] = (a0 * p2[0] + a1 * p2[1] + a2 * p2[2]) * inv;
+  const double B = (a0 * b[0] + a1 * b[1] + a2 * b[2]) * inv;
+  const double S = (a0 * s[0] + a1 * s[1] + a2 * s[2]) * inv;
+  const double y = 0.5 - o->xi3[0];
+  const double side = fma(1.0 / 30.0, S, u[2]);       // y^2 / 2 - 1/24 = 1/30
+  out[0] = fma(-y, B, side);
+  out[1] = fma(-1.0 / 24.0, S, u[2]);
+  out[2] = fma(y, B, side);
 }
 
 // FP32 form of weno3 (mixed precision).  (sigma_k + eps)^8 underflows in FP32
