@@ -189,6 +189,20 @@ struct NoAlloc {
   }
 };
 
+// The operator table of degree N, built once per process (initialisation of a
+// function-local static is thread safe).  Its long double arithmetic is
+// binary128 in software on Arm: 0.55 ms, as long as the update of 146 patches
+// of 2D N = 5 on the GPU, and the table is a constant of the degree.
+template <int N>
+const Ops& degree_ops() {
+  static const Ops table = [] {
+    Ops o;
+    build_ops(N, &o);
+    return o;
+  }();
+  return table;
+}
+
 template <int D, int N>
 int run_noalloc(unsigned char* base, double gamma, const double* h, double dt, const double* patches,
                 int count, double* vnew, double* faces, cudaStream_t s, char* err, size_t errlen) {
@@ -204,8 +218,7 @@ int run_noalloc(unsigned char* base, double gamma, const double* h, double dt, c
     return ADG_ERR_CAPACITY;
   }
   Upload up;
-  Ops& ops_host = *reinterpret_cast<Ops*>(up.bytes + PARAMS_BYTES);
-  build_ops(N, &ops_host);
+  memcpy(up.bytes + PARAMS_BYTES, &degree_ops<N>(), sizeof(Ops));
   Params* params_dev = reinterpret_cast<Params*>(base + CTRL_BYTES);
   Ops* ops_dev = reinterpret_cast<Ops*>(base + CTRL_BYTES + PARAMS_BYTES);
   Params p;
