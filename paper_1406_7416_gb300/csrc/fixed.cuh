@@ -119,4 +119,34 @@ __device__ __forceinline__ double fx_double(long long R, int b) {
   return __hiloint2double((int)(oh | (s & 0x80000000u)), (int)ol);
 }
 
+// ROWS outputs of an operator on the line x: out(a, sum_j m[a n + j] x[j]) for
+// a < ROWS, m of scale exponent g.  Lines out of the range are settled by a
+// branch: zero, or NaN in every output (as a line with a NaN or an infinity
+// has in FP64, up to the sign of an infinity).
+template <int n, int ROWS, typename Out>
+__device__ __forceinline__ void fx_apply(const double* x, const FxOp* __restrict__ m, int g, Out out) {
+  unsigned key = 0;
+#pragma unroll
+  for (int j = 0; j < n; ++j) key = max(key, fx_key(x[j]));
+  const unsigned e = key >> 21;
+  const int b = (int)e + g + 5;
+  if (e >= FX_E_MIN && e < FX_E_MAX && b >= 70 && b <= 2040) {
+    FxVal f[n];
+#pragma unroll
+    for (int j = 0; j < n; ++j) f[j] = fx_val(x[j], e);
+    constexpr int U = ROWS < 2 ? 1 : 2;
+#pragma unroll U
+    for (int a = 0; a < ROWS; ++a) {
+      FxAcc acc;
+#pragma unroll
+      for (int j = 0; j < n; ++j) acc.add(f[j], m[a * n + j]);
+      out(a, fx_double(acc.sum(), b));
+    }
+  } else {
+    const double fill = (e < FX_E_MIN || b < 70) ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+#pragma unroll 1
+    for (int a = 0; a < ROWS; ++a) out(a, fill);
+  }
+}
+
 }  // namespace adg

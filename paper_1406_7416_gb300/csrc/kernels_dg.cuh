@@ -6,6 +6,7 @@
 #include <climits>
 
 #include "adg_internal.h"
+#include "fixed.cuh"
 
 namespace adg {
 
@@ -113,6 +114,73 @@ __device__ __forceinline__ void picard_time(T* __restrict__ q, const UT* __restr
       for (int j = 0; j < n; ++j) acc += Kt[m * n + j] * Sl[j];
       q[v * NST + i + m * ND] = u0 - acc;
     }
+  }
+}
+
+// FP64 sweep phases with the contractions on the integer pipes (fixed.cuh).  The
+// FP64 pipe bounds an FP64 sweep: per node its fluxes take 16 operations in 2D
+// and a division, its contractions (D + 1) n + D + 1 per variable, more than
+// four times as many at n = 6.  The FP64 pipe keeps the fluxes and the sums over
+// the axes; the phases run by lines, each line read and converted once for its
+// n outputs, and the derivative phase works in place, so that the axes need no
+// barrier between them.  Measured (GB300, predictor phase per step): 256^2
+// N = 5 FP64 17.1 -> 6.7 ms, 67 x 53 N = 6 FP64 1.93 -> 0.73 ms, 33 x 29 x 30
+// N = 3 FP64 7.75 -> 3.19 ms, 200^2 N = 9 mixed (nine FP32 sweeps and this one)
+// 17.0 -> 11.1 ms.
+//
+// Fluxes of `nodes` space-time nodes (all NST, or the ND of time node 0).
+template <int D, int n>
+__device__ __forceinline__ void flux_fx(const double* __restrict__ q, double* __restrict__ F, double gm1,
+                                        int nodes, int qstride, int tid, int nth) {
+  constexpr int NV = D + 2, NST = ipow(n, D + 1);
+  for (int l = tid; l < nodes; l += nth) {
+    double Q[NV], Fl[D][D + 2];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Q[v] = q[v * qstride + l];
+    euler_fluxes_sym<D>(Q, gm1, Fl);
+#pragma unroll
+    for (int k = 0; k < D; ++k)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) F[(k * NV + v) * NST + l] = Fl[k][v];
+  }
+}
+
+// Derivative phase, F_k <- (c_k D) x_k F_k in place for every axis: one thread
+// per line of n nodes (cD[k n n ..] is c_k D with scale exponent gD[k]).  NL
+// lines per variable (those of all time nodes, or of time node 0).
+template <int D, int n, int NL>
+__device__ __forceinline__ void deriv_fx(double* F, const FxOp* cD, const int* gD, int tid, int nth) {
+  constexpr int NV = D + 2, NST = ipow(n, D + 1);
+  for (int e = tid; e < D * NV * NL; e += nth) {
+    const int kv = e / NL, r = e - kv * NL;
+    const int k = kv / NV;
+    const int st = (k == 0) ? 1 : (k == 1 ? n : n * n);
+    double* f = F + kv * NST + n * r - (n - 1) * (r % st);
+    double x[n];
+#pragma unroll
+    for (int j = 0; j < n; ++j) x[j] = f[j * st];
+    fx_apply<n, n>(x, cD + k * (n * n), gD[k], [&](int a, double y) { f[a * st] = y; });
+  }
+}
+
+// Time phase, q <- u - Ktau S with S = sum_k of the derivative phase's F_k.
+template <int D, int n>
+__device__ __forceinline__ void time_fx(const double* F, double* q, const double* u, const FxOp* Kt,
+                                        int gK, int tid, int nth) {
+  constexpr int NV = D + 2, ND = ipow(n, D), NST = ipow(n, D + 1);
+  for (int e = tid; e < NV * ND; e += nth) {
+    const int v = e / ND, i = e - v * ND;
+    double S[n];
+#pragma unroll
+    for (int m = 0; m < n; ++m) {
+      double s = F[v * NST + i + m * ND];
+#pragma unroll
+      for (int k = 1; k < D; ++k) s += F[(k * NV + v) * NST + i + m * ND];
+      S[m] = s;
+    }
+    const double u0 = u[e];
+    double* qv = q + v * NST + i;
+    fx_apply<n, n>(S, Kt, gK, [&](int m, double y) { qv[m * ND] = u0 - y; });
   }
 }
 
@@ -426,8 +494,9 @@ __device__ __forceinline__ int trace_index(int e, int& base, int& stk, int& s) {
 template <int D, int N, bool MIXED>
 __host__ __device__ constexpr size_t predictor_smem_bytes() {
   using DM = Dims<D, N>;
+  // u, q, F, fbar, the operators of PredOps and (split final stage) Mvol, w, phi
   size_t d = (size_t)DM::NV * DM::ND + (size_t)DM::NV * DM::NST + (size_t)D * DM::NV * DM::NST +
-             (size_t)D * DM::NV * DM::ND + 3 * DM::n * DM::n + 3 * DM::n;
+             (size_t)D * DM::NV * DM::ND + (2 * D + 1) * DM::n * DM::n + 4 * DM::n + 3 * DM::n;
   // the FP32 sweep arrays qf, Ff live inside the FP64 flux array F (unused
   // until the FP32 sweeps are over); u and the trace weights in FP32 stay
   // apart (the FP32 sweep operators are in constant memory)
@@ -445,10 +514,15 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
   double* q = u + NV * ND;
   double* F = q + NV * NST;
   double* fbar = F + D * NV * NST;
-  double* Dm = fbar + D * NV * ND;
-  double* Kt = Dm + n * n;
-  double* Mv = Kt + n * n;
-  double* w = Mv + n * n;
+  // integer-pipe operators: c_k D and c_k Mvol per axis (of the state in hand),
+  // Ktau, its row sums, the time weights and the two traces
+  FxOp* cD = reinterpret_cast<FxOp*>(fbar + D * NV * ND);
+  FxOp* cM = cD + D * n * n;
+  FxOp* Ktx = cM + D * n * n;
+  FxOp* kapx = Ktx + n * n;         // row sums of Ktau
+  FxOp* wx = kapx + n;
+  FxOp* phx = wx + n;               // [2][n]
+  double* w = reinterpret_cast<double*>(phx + 2 * n);
   double* ph0 = w + n;
   double* ph1 = ph0 + n;
   // FP32 sweep arrays inside F: (1 + D) NV NST floats fit in D NV NST doubles
@@ -457,14 +531,11 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
   float* uf = reinterpret_cast<float*>(ph1 + n);
   float* ph0f = uf + NV * ND;
   float* ph1f = ph0f + n;
+  __shared__ double s_rs[5];        // largest row sums: D, Mvol, Ktau, w, phi
+  __shared__ int gD[3], gM[3];      // scale exponents of cD, cM
 
   const int tid = threadIdx.x, nth = blockDim.x;
   const Ops* o = bt.pps[0]->ops;      // every state of a batch has degree N
-  for (int i = tid; i < n * n; i += nth) {
-    Dm[i] = o->D[i];
-    Kt[i] = o->Kt[i];
-    Mv[i] = o->Mvol[i];
-  }
   for (int i = tid; i < n; i += nth) {
     w[i] = o->w[i];
     ph0[i] = o->phi0[i];
@@ -474,6 +545,35 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
       ph1f[i] = (float)o->phi1[i];
     }
   }
+  if (tid < 32) {
+    double rs[5] = {};
+    if (tid < n) {
+      for (int j = 0; j < n; ++j) {
+        rs[0] += fabs(o->D[tid * n + j]);
+        rs[1] += fabs(o->Mvol[tid * n + j]);
+        rs[2] += fabs(o->Kt[tid * n + j]);
+        rs[3] += fabs(o->w[j]);
+        rs[4] += fabs(tid & 1 ? o->phi1[j] : o->phi0[j]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 5; ++r) {
+      for (int d = 16; d > 0; d >>= 1) rs[r] = fmax(rs[r], __shfl_xor_sync(0xffffffffu, rs[r], d));
+      if (tid == 0) s_rs[r] = rs[r];
+    }
+  }
+  __syncthreads();
+  const int gK = fx_scale(s_rs[2]), gw = fx_scale(s_rs[3]), gph = fx_scale(s_rs[4]);
+  for (int i = tid; i < n * n; i += nth) Ktx[i] = fx_op(o->Kt[i], gK);
+  for (int i = tid; i < n; i += nth) {
+    double ks = 0.0;
+    for (int j = 0; j < n; ++j) ks += o->Kt[i * n + j];
+    kapx[i] = fx_op(ks, gK);
+    wx[i] = fx_op(o->w[i], gw);
+    phx[i] = fx_op(o->phi0[i], gph);
+    phx[n + i] = fx_op(o->phi1[i], gph);
+  }
+  int state = -1;
   for (long long g = blockIdx.x; g < bt.pre[bt.n]; g += gridDim.x) {
     const int sidx = batch_state(bt, g);
     const Params& p = *bt.pps[sidx];
@@ -486,6 +586,20 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
     const double gm1 = p.gamma - 1.0;
     const double* Uc = p.b.U[p.cur] + cell * (NV * ND);
     for (int i = tid; i < NV * ND; i += nth) u[i] = Uc[i];
+    if (sidx != state) {
+      // the operators of this state's step, scaled by c_k
+      state = sidx;
+      if (tid < D) {
+        gD[tid] = fx_scale(p.b.coef[tid] * s_rs[0]);
+        gM[tid] = fx_scale(p.b.coef[tid] * s_rs[1]);
+      }
+      for (int i = tid; i < D * n * n; i += nth) {
+        const int k = i / (n * n), r = i - k * (n * n);
+        const double ck = p.b.coef[k];
+        cD[i] = fx_op(ck * o->D[r], fx_scale(ck * s_rs[0]));
+        cM[i] = fx_op(ck * o->Mvol[r], fx_scale(ck * s_rs[1]));
+      }
+    }
     __syncthreads();
     int it0 = 0;
     const int n32 = p.iters - p.fp64_sweeps;    // sweeps in FP32
@@ -516,21 +630,34 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
         __syncthreads();
       }
       if (!last64)
-        for (int e = tid; e < NV * NST; e += nth) q[e] = (double)qf[e];
+        for (int e = tid; e < NV * NST; e += nth) q[e] = widen_f32(qf[e]);
       it0 = n32;
     } else {
-      for (int e = tid; e < NV * NST; e += nth) {
-        const int v = e / NST, l = e - v * NST;
-        q[e] = u[v * ND + (l % ND)];
+      // the first sweep starts from u (x) 1, whose fluxes and derivatives S are
+      // the same at every time node: it runs on the n^d spatial nodes, and
+      // q_m = u - kappa_m S with kappa = Ktau 1
+      flux_fx<D, n>(u, F, gm1, ND, ND, tid, nth);
+      __syncthreads();
+      deriv_fx<D, n, ND / n>(F, cD, gD, tid, nth);
+      __syncthreads();
+      for (int e = tid; e < NV * ND; e += nth) {
+        const int v = e / ND, i = e - v * ND;
+        double S = F[v * NST + i];
+#pragma unroll
+        for (int k = 1; k < D; ++k) S += F[(k * NV + v) * NST + i];
+        const double u0 = u[e];
+        double* qv = q + v * NST + i;
+        fx_apply<1, n>(&S, kapx, gK, [&](int m, double y) { qv[m * ND] = u0 - y; });
       }
+      it0 = 1;
     }
     __syncthreads();
     for (int it = it0; it < p.iters; ++it) {
-      picard_flux<D, n, double>(q, F, gm1, tid, nth);
+      flux_fx<D, n>(q, F, gm1, NST, NST, tid, nth);
       __syncthreads();
-      picard_deriv<D, n, double>(F, q, Dm, c, tid, nth);
+      deriv_fx<D, n, NST / n>(F, cD, gD, tid, nth);
       __syncthreads();
-      picard_time<D, n, double>(q, u, Kt, tid, nth);
+      time_fx<D, n>(F, q, u, Ktx, gK, tid, nth);
       __syncthreads();
     }
     if (split) {
@@ -592,47 +719,53 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
         for (int m = 0; m < n; ++m) acc += dF[kv * NST + i + m * ND];
         fbar[e] += (double)acc;
       }
+      __syncthreads();
     } else {
       // corrector volume term from the time-averaged nodal fluxes
-      picard_flux<D, n, double>(q, F, gm1, tid, nth);
+      flux_fx<D, n>(q, F, gm1, NST, NST, tid, nth);
       __syncthreads();
       for (int e = tid; e < D * NV * ND; e += nth) {
         const int kv = e / ND, i = e - kv * ND;
-        double acc = 0.0;
+        double x[n];
 #pragma unroll
-        for (int m = 0; m < n; ++m) acc += w[m] * F[kv * NST + i + m * ND];
-        fbar[e] = acc;
+        for (int m = 0; m < n; ++m) x[m] = F[kv * NST + i + m * ND];
+        fx_apply<n, 1>(x, wx, gw, [&](int, double y) { fbar[e] = y; });
       }
+      __syncthreads();
     }
+    // c_k Mvol x_k fbar_k in place, by lines, then the sum with u
+    for (int e = tid; e < D * NV * NF; e += nth) {
+      const int kv = e / NF, r = e - kv * NF;
+      const int k = kv / NV;
+      const int st = (k == 0) ? 1 : (k == 1 ? n : n * n);
+      double* f = fbar + kv * ND + n * r - (n - 1) * (r % st);
+      double x[n];
+#pragma unroll
+      for (int j = 0; j < n; ++j) x[j] = f[j * st];
+      fx_apply<n, n>(x, cM + k * (n * n), gM[k], [&](int a, double y) { f[a * st] = y; });
+    }
+    // space-time traces on the faces, trace[cell][k][side][v][ts + NF * m], by
+    // lines: the n nodes of a line along axis k give both faces normal to k, and
+    // the line's index within its variable is the trace's index ts + NF m
+    if (!split)
+      for (int e = tid; e < D * NV * NT; e += nth) {
+        const int k = e / (NV * NT), vr = e - k * (NV * NT);
+        const int st = (k == 0) ? 1 : (k == 1 ? n : n * n);
+        const double* f = q + n * vr - (n - 1) * (vr % st);
+        double x[n];
+#pragma unroll
+        for (int j = 0; j < n; ++j) x[j] = f[j * st];
+        double* t = tr + (2 * k) * (NV * NT) + vr;
+        fx_apply<n, 2>(x, phx, gph, [&](int side, double y) { t[side * (NV * NT)] = y; });
+      }
     __syncthreads();
     double* Uo = p.b.U[1 - p.cur] + cell * (NV * ND);
     for (int e = tid; e < NV * ND; e += nth) {
-      const int v = e / ND, i = e - v * ND;
       double acc = u[e];
 #pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const int st = (k == 0) ? 1 : (k == 1 ? n : n * n);
-        const int ak = (i / st) % n;
-        const double* f = fbar + (k * NV + v) * ND + (i - ak * st);
-        double t = 0.0;
-#pragma unroll
-        for (int j = 0; j < n; ++j) t += Mv[ak * n + j] * f[j * st];
-        acc += c[k] * t;
-      }
+      for (int k = 0; k < D; ++k) acc += fbar[k * (NV * ND) + e];
       Uo[e] = acc;
     }
-    // space-time traces on the 2D faces: trace[cell][k][side][v][ts + NF * m]
-    if (!split)
-      for (int e = tid; e < D * 2 * NV * NT; e += nth) {
-        int base, stk, s;
-        const int v = trace_index<D, n>(e, base, stk, s);
-        const double* ph = s ? ph1 : ph0;
-        const double* qq = q + v * NST + base;
-        double acc = 0.0;
-#pragma unroll
-        for (int a = 0; a < n; ++a) acc += ph[a] * qq[a * stk];
-        tr[e] = acc;
-      }
     __syncthreads();
   }
 }
