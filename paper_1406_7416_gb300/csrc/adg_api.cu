@@ -304,6 +304,7 @@ int ensure_allocated(adg_state* st) {
   ALLOC(st->d_pre1, long long, 20);
   ALLOC(st->d_dts1, double, 1);
   ALLOC(b.patch, double, chunk * parts[0]);
+  ALLOC(b.nbr, int, chunk * 2 * st->dim);
   ALLOC(b.sweep[0], double, chunk * parts[1]);
   ALLOC(b.sweep[1], double, chunk * parts[2]);
   if (st->dim == 3) ALLOC(b.sweep[2], double, chunk * parts[3]);

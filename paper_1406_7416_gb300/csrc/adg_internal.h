@@ -99,6 +99,7 @@ struct Bufs {
   uint8_t* vok;          // [cells] 1 where vstar is P of the cell's current DOFs
   // limiter scratch, sized for one chunk of `chunk` troubled cells
   double* patch;         // [chunk][nv][L^d]
+  int* nbr;              // [chunk][2 d] the pass's position of each face neighbour, -1: not in it
   double* sweep[3];      // [chunk][nv][...] after the x, y, z reconstructions
   double* qsub;          // [chunk][(Ns+2)^d][nv][3^(d+1)]
   double* fsub[3];       // [chunk][nv][faces along axis k]
