@@ -255,9 +255,9 @@ struct Launch {
           if constexpr (D == 3) {
             static_assert(SubTraces<N>::per_cell <= 2LL * DM::NED * DM::NV * DM::NST3,
                           "the traces fit the subcell predictor's scratch");
-            static const int gw = persistent_grid(k_lim_predict_s3<N>, 256, 0, 1LL << 40);
-            const long long want = (ncross + 7) / 8;
-            k_lim_predict_s3<N><<<(int)(want < gw ? want : gw), 256, 0, s>>>(lim);
+            static const int gw = persistent_grid(k_lim_predict_s3<N>, 128, 0, 1LL << 40);
+            const long long want = (ncross + 3) / 4;
+            k_lim_predict_s3<N><<<(int)(want < gw ? want : gw), 128, 0, s>>>(lim);
           }
         } else {
           constexpr int W = LimWarps<D>::W;
