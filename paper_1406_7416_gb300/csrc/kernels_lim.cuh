@@ -1562,6 +1562,192 @@ __global__ void __launch_bounds__(256) k_lim_flux(Batch bt, int pass) {
   }
 }
 
+// L5 in FP64: the same sub-face fluxes from FP64 nodal values, one lane per
+// point (3D: the 27 points of one sub-face; 2D: the 9 of each of three), so
+// that a warp reads a subcell's nodal values together.  A warp takes a few
+// rounds of sub-faces and then adds their points, one lane per (sub-face,
+// variable) in point order: added after each sub-face, the sums would be 26
+// dependent FP64 operations on five lanes.
+//
+// The FP64 pipe bounds this kernel (88% busy in the thread-per-sub-face form,
+// 107 operations per point in 3D): the traces, 30 of them, go to the integer
+// pipes (fixed.cuh), and with the Rusanov flux each side's flux and the
+// dissipation enter the point's value by FMAs with its weight folded in
+// instead of being formed first (27 operations instead of 35), the larger
+// speed by an integer comparison.
+//
+// Measured (GB300): 33 x 29 x 30 N = 3, 5611 troubled cells, 12.4 -> 10.8 ms
+// per axis (84% FP64 pipe, 75 operations per point); 2D N = 5, 146 patches,
+// 72 -> 42 us per axis.
+template <int D>
+struct FluxPoints {
+  static constexpr int SPR = D == 3 ? 1 : 3;            // sub-faces per round
+  static constexpr int ROUNDS = D == 3 ? 6 : 2;         // 30 or 24 sums of a turn, one per lane
+  static constexpr int FACES = SPR * ROUNDS;            // sub-faces of one warp's turn
+};
+
+template <int D, int N, int k, bool OSHER>
+__global__ void __launch_bounds__(128) k_lim_flux_d(Batch bt, int pass) {
+  pass = lim_pass(bt, pass);
+  using DM = Dims<D, N>;
+  using FP = FluxPoints<D>;
+  constexpr int NV = DM::NV, NST3 = DM::NST3, ND3 = DM::ND3, NE = DM::NE, NED = DM::NED, Ns = DM::Ns;
+  constexpr int NFK = (Ns + 1) * DM::NSF;
+  constexpr int stk = (k == 0) ? 1 : (k == 1 ? 3 : 9);    // node stride of axis k
+  __shared__ FxOp ph[2][3];         // the traces at the high and low ends
+  __shared__ double hw[ND3];        // half the weight of each point
+  __shared__ double s_pt[4][FP::FACES * NV][ND3 + 1];
+  __shared__ int s_g;
+  const Ops* o = bt.pps[0]->ops;
+  if (threadIdx.x < 32) {
+    const int i = threadIdx.x;
+    double s0 = 0.0, s1 = 0.0;
+    for (int q = 0; q < 3; ++q) {
+      s0 += fabs(o->phi03[q]);
+      s1 += fabs(o->phi13[q]);
+    }
+    const int g = fx_scale(fmax(s0, s1));
+    if (i < 6) ph[i / 3][i % 3] = fx_op(i < 3 ? o->phi13[i] : o->phi03[i - 3], g);
+    if (i == 0) s_g = g;
+    if (i < ND3) hw[i] = 0.5 * o->w3[i % 3] * o->w3[(i / 3) % 3] * (D == 3 ? o->w3[i / 9] : 1.0);
+  }
+  __syncthreads();
+  const int g = s_g;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int pl = lane < 27 ? lane : 26;                   // idle lanes mirror lane 26
+  const int fi = pl / ND3, t = pl - fi * ND3;
+  // first node of the point's line: its digits over the tangential axes, then
+  // the time node
+  const int m = D == 3 ? t / 9 : t / 3;
+  const int d0 = t % 3, d1 = D == 3 ? (t / 3) % 3 : 0;
+  const int base = m * ND3 + (k == 0 ? 3 * d0 + 9 * d1 : (k == 1 ? d0 + 9 * d1 : d0 + 3 * d1));
+  const double h = hw[t];
+  const long long total = bt.pre[bt.n] * NFK;
+  const long long turns = (total + FP::FACES - 1) / FP::FACES;
+  for (long long turn = (long long)blockIdx.x * 4 + w; turn < turns; turn += (long long)gridDim.x * 4) {
+#pragma unroll 1
+    for (int rd = 0; rd < FP::ROUNDS; ++rd) {
+      const int ff = rd * FP::SPR + fi;
+      const long long f = turn * FP::FACES + ff;
+      if (turn * FP::FACES + rd * FP::SPR >= total) break;     // (uniform over the warp)
+      const long long fe = f < total ? f : total - 1;
+      const long long tg = fe / NFK;
+      const LimItem it = lim_item(bt, tg);
+      const Params& p = *bt.pps[it.s];
+      const long long j = it.j;
+      int fck = 0, sl = 0, sr = 0;
+      {
+        int r = (int)(fe - tg * NFK), mul = 1;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+          const int ext = (a == k) ? Ns + 1 : Ns;
+          const int c = r % ext;
+          r /= ext;
+          if (a == k) fck = c;
+          // left / right subcells in the (Ns+2)^d block (array index = local + 1)
+          sl += ((a == k) ? c : c + 1) * mul;
+          sr += (c + 1) * mul;
+          mul *= NE;
+        }
+      }
+      int wall = 0;                          // -1: low wall (ghost left), +1: high wall (ghost right)
+      long long jL = j, jR = j;
+      if (fck == 0 || fck == Ns) {
+        // the ghost's side from the neighbour that computed it as its interior
+        const int j2 = shared_neighbour<D>(p, j, k, fck == 0 ? -1 : 1);
+        constexpr int across = Ns * ((k == 0) ? 1 : (k == 1 ? NE : NE * NE));
+        if (j2 >= 0 && fck == 0) {
+          jL = j2;
+          sl += across;
+        } else if (j2 >= 0) {
+          jR = j2;
+          sr -= across;
+        }
+        // reflecting walls: as in k_lim_flux
+        const int side = fck == 0 ? 0 : 1;
+        if (p.geo.bc[2 * k + side] == ADG_BC_REFLECTIVE) {
+          const long long cell = p.b.list[1 - p.cur][pass * p.chunk + j];
+          int ijk[3];
+          cell_coords<D>(cell, p.geo, ijk);
+          if (side == 0 && ijk[k] == 0) wall = -1;
+          if (side == 1 && ijk[k] == p.geo.n[k] - 1) wall = 1;
+        }
+      }
+      const double* qL = p.b.qsub + (jL * NED + sl) * (size_t)(NV * NST3) + base;
+      const double* qR = p.b.qsub + (jR * NED + sr) * (size_t)(NV * NST3) + base;
+      double QL[NV], QR[NV], G[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const double* a = qL + v * NST3;
+        const double* b = qR + v * NST3;
+        const double xa[3] = {a[0], a[stk], a[2 * stk]}, xb[3] = {b[0], b[stk], b[2 * stk]};
+        fx_apply<3, 1>(xa, ph[0], g, [&](int, double y) { QL[v] = y; });
+        fx_apply<3, 1>(xb, ph[1], g, [&](int, double y) { QR[v] = y; });
+      }
+      if (wall < 0) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) QL[v] = QR[v];
+        QL[1 + k] = -QR[1 + k];
+      } else if (wall > 0) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) QR[v] = QL[v];
+        QR[1 + k] = -QL[1 + k];
+      }
+      if constexpr (OSHER) {
+        face_flux<D>(ADG_FLUX_OSHER, QL, QR, k, p.gamma, G);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) G[v] *= 2.0 * h;
+      } else {
+        // h (F_k(QL) + F_k(QR) - s (QR - QL)), s the larger |v_k| + c (as bits:
+        // not negative, and a NaN of either sign is above every number)
+        const double gm1 = p.gamma - 1.0;
+        unsigned long long s = 0;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) G[v] = 0.0;
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+          const double* Q = side ? QR : QL;
+          const double r = 1.0 / Q[0];
+          double kin = 0.0;
+#pragma unroll
+          for (int a = 0; a < D; ++a) kin += Q[1 + a] * Q[1 + a];
+          const double pr = gm1 * (Q[D + 1] - 0.5 * kin * r);
+          const double vk = Q[1 + k] * r, hv = h * vk;
+          G[0] += h * Q[1 + k];
+#pragma unroll
+          for (int a = 0; a < D; ++a) G[1 + a] += hv * Q[1 + a];
+          G[1 + k] += h * pr;
+          G[D + 1] += hv * (Q[D + 1] + pr);
+          const double sp = fabs(vk) + sqrt(p.gamma * pr * r);
+          const unsigned long long b = (unsigned long long)__double_as_longlong(sp);
+          s = b > s ? b : s;
+        }
+        const double hs = h * __longlong_as_double((long long)s);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) G[v] -= hs * (QR[v] - QL[v]);
+      }
+      if (lane < 27) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) s_pt[w][ff * NV + v][t] = G[v];
+      }
+    }
+    __syncwarp();
+    for (int q = lane; q < FP::FACES * NV; q += 32) {
+      const int ff = q / NV, v = q - ff * NV;
+      const long long f = turn * FP::FACES + ff;
+      if (f < total) {
+        const long long tg = f / NFK;
+        const LimItem it = lim_item(bt, tg);
+        double acc = s_pt[w][q][0];
+#pragma unroll
+        for (int i = 1; i < ND3; ++i) acc += s_pt[w][q][i];
+        bt.pps[it.s]->b.fsub[k][((size_t)it.j * NV + v) * NFK + (int)(f - tg * NFK)] = acc;
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // L6: finite volume update, storage of v^{n+1}, reconstruction R, per-cell
 // min/max and wave speed, sub-face fluxes of the cell faces, and marking of
 // unlimited face neighbours for the flux correction.  One block per cell.

@@ -214,6 +214,25 @@ struct Launch {
     k_lim_predict_i<D, N, WT><<<(int)(want < gw ? want : gw), 128, 0, s>>>(lim);
   }
 
+  // The FP64 sub-face fluxes of at most `ch` troubled cells, persistent.
+  template <int K, bool OSHER>
+  static void launch_flux_axis(const Batch& lim, int pass, long long want, cudaStream_t s) {
+    static const int gw = persistent_grid(k_lim_flux_d<D, N, K, OSHER>, 128, 0, 1LL << 40);
+    k_lim_flux_d<D, N, K, OSHER><<<(int)(want < gw ? want : gw), 128, 0, s>>>(lim, pass);
+  }
+  static void launch_flux_d(const Batch& lim, int pass, long long ch, int flux, cudaStream_t s) {
+    const long long want = (ch * (Ns + 1) * DM::NSF / FluxPoints<D>::FACES + 4) / 4;
+    if (flux == ADG_FLUX_OSHER) {
+      launch_flux_axis<0, true>(lim, pass, want, s);
+      launch_flux_axis<1, true>(lim, pass, want, s);
+      if constexpr (D == 3) launch_flux_axis<2, true>(lim, pass, want, s);
+    } else {
+      launch_flux_axis<0, false>(lim, pass, want, s);
+      launch_flux_axis<1, false>(lim, pass, want, s);
+      if constexpr (D == 3) launch_flux_axis<2, false>(lim, pass, want, s);
+    }
+  }
+
   // One limiter pass (pass < 0: the pass of the device-sized loop).
   static cudaError_t lim_pass(const StepLaunch& sl, int pass, cudaStream_t s) {
     cudaError_t e;
@@ -314,9 +333,7 @@ struct Launch {
       k_lim_flux<D, N, 1, double, float><<<gf, 256, 0, s>>>(lim, pass);
       if (D == 3) k_lim_flux<D, N, (D == 3 ? 2 : 1), double, float><<<gf, 256, 0, s>>>(lim, pass);
     } else {
-      k_lim_flux<D, N, 0, double, double><<<gf, 256, 0, s>>>(lim, pass);
-      k_lim_flux<D, N, 1, double, double><<<gf, 256, 0, s>>>(lim, pass);
-      if (D == 3) k_lim_flux<D, N, (D == 3 ? 2 : 1), double, double><<<gf, 256, 0, s>>>(lim, pass);
+      launch_flux_d(lim, pass, ch, sl.flux, s);
     }
     k_lim_update<D, N><<<(int)(ch < kNumSM * 8 ? ch : kNumSM * 8), 128, cell_smem(), s>>>(lim, pass);
     return cudaGetLastError();

@@ -160,11 +160,7 @@ struct NoAlloc {
       k_lim_sweep<D, N, (D == 3 ? 2 : 1), double><<<grid_for(ch * DM::NV * DM::LD, 256), 256, 0, s>>>(lim, 0);
     const long long ncross = ch * (DM::NSD + 2 * D * DM::NSF);
     Launch<D, N>::template launch_predict_i<double>(lim, ncross, s);
-    k_lim_flux<D, N, 0, double, double><<<grid_for(ch * (DM::Ns + 1) * DM::NSF, 256), 256, 0, s>>>(lim, 0);
-    k_lim_flux<D, N, 1, double, double><<<grid_for(ch * (DM::Ns + 1) * DM::NSF, 256), 256, 0, s>>>(lim, 0);
-    if (D == 3)
-      k_lim_flux<D, N, (D == 3 ? 2 : 1), double, double><<<grid_for(ch * (DM::Ns + 1) * DM::NSF, 256), 256, 0, s>>>(
-          lim, 0);
+    Launch<D, N>::launch_flux_d(lim, 0, ch, ADG_FLUX_RUSANOV, s);
     k_noalloc_write<D, N><<<grid_for(ch * DM::NV * DM::NSD, 256), 256, 0, s>>>(p, count, vnew, faces);
     return cudaGetLastError();
   }
