@@ -14,6 +14,12 @@ constexpr int MAXNS = 19;             // subcells per axis, Ns = 2N + 1 <= 19
 constexpr double WENO_EPS = 1e-14;    // WENO3 weights: lambda_k / (sigma_k + eps)^8
 constexpr double WENO_LAMBDA_C = 1e5; // central stencil; side stencils use 1
 
+// An operator entry v 2^(g - 63) of a fixed-point contraction (fixed.cuh),
+// v = h 2^32 + l with l signed, g the operator's scale exponent.
+struct FxOp {
+  int h, l;
+};
+
 // 1D operators of the degree-N nodal Gauss-Legendre basis on [0, 1] and of the
 // degree-2 subcell basis, generated on the host (ops_host.cpp) and copied to
 // the device once per state.
@@ -45,6 +51,9 @@ struct Ops {
   // averages, Wf[k][node * 3 + r] = sum_p E[node][p] C[k][p][r]
   float Cf[3][6];
   float Wf[3][9];
+  // P1 and R1 for the integer pipes (fixed.cuh), with their scale exponents
+  FxOp P1x[MAXNS * MAXN], R1x[MAXN * MAXNS];
+  int gP1, gR1;
 };
 
 // Builds the operator table of degree N (host, long double arithmetic).

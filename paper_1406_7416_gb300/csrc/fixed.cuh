@@ -21,12 +21,9 @@
 
 #include <stdint.h>
 
-namespace adg {
+#include "adg_internal.h"
 
-// An operator entry v 2^(g - 63), v = h 2^32 + l with l signed.
-struct FxOp {
-  int h, l;
-};
+namespace adg {
 
 // A data element on its line's scale, f = h 2^32 + l with l signed, |f| < 2^59.
 struct FxVal {

@@ -427,7 +427,7 @@ __device__ __forceinline__ void apply_pass_ct(const T* __restrict__ in, T* __res
   }
 }
 
-template <int D, int NV, int NI, int NO, typename T = double>
+template <int D, int NV, int NI, int NO, typename T>
 __device__ __forceinline__ T* apply_ct(T* a, T* b, const T* M, int tid, int nth) {
   apply_pass_ct<D, NV, NI, NO, 0, T>(a, b, M, tid, nth);
   __syncthreads();
@@ -437,6 +437,59 @@ __device__ __forceinline__ T* apply_ct(T* a, T* b, const T* M, int tid, int nth)
   if (D == 2) return a;
   apply_pass_ct<D, NV, NI, NO, 2, T>(a, b, M, tid, nth);
   __syncthreads();
+  return b;
+}
+
+// The FP64 operator of a projection or reconstruction: its fixed-point entries
+// (shared memory) with their scale exponent, and its doubles.
+struct FxMat {
+  const FxOp* x;
+  int g;
+  const double* d;
+};
+
+// One pass of apply_ct in FP64 on the integer pipes (fixed.cuh): one thread per
+// line of NI points along axis K.  Lines of two points (N = 1) stay on the FP64
+// pipe: the conversions cost more there than the two FMAs of each output (and
+// at N = 3 already half of the FMAs').
+template <int D, int NV, int NI, int NO, int K>
+__device__ __forceinline__ void apply_pass_fx(const double* in, double* out, const FxMat& M, int tid,
+                                              int nth) {
+  if constexpr (NI < 3) {
+    apply_pass_ct<D, NV, NI, NO, K, double>(in, out, M.d, tid, nth);
+  } else {
+    constexpr int I0 = (0 < K) ? NO : NI, I1 = (D < 2) ? 1 : ((1 < K) ? NO : NI), I2 = (D < 3) ? 1 : NI;
+    constexpr int ISZ = I0 * I1 * I2, LINES = ISZ / NI, OSZ = LINES * NO;
+    constexpr int S = (K == 0) ? 1 : (K == 1 ? I0 : I0 * I1);     // stride along K, in and out
+    for (int e = tid; e < NV * LINES; e += nth) {
+      const int v = e / LINES, r = e - v * LINES;
+      const int lo = r % S, hi = r / S;                           // places below and above axis K
+      const double* src = in + v * ISZ + lo + hi * (S * NI);
+      double* dst = out + v * OSZ + lo + hi * (S * NO);
+      double x[NI];
+#pragma unroll
+      for (int j = 0; j < NI; ++j) x[j] = src[j * S];
+      fx_apply<NI, NO>(x, M.x, M.g, [&](int a, double y) { dst[a * S] = y; });
+    }
+  }
+}
+
+// Tensor projection / reconstruction in FP64 through two buffers, by a block
+// or (WARP) a warp.
+template <int D, int NV, int NI, int NO, bool WARP = false>
+__device__ __forceinline__ double* apply_fx(double* a, double* b, const FxMat& M, int tid, int nth) {
+  auto sync = [] {
+    if (WARP) __syncwarp();
+    else __syncthreads();
+  };
+  apply_pass_fx<D, NV, NI, NO, 0>(a, b, M, tid, nth);
+  sync();
+  if (D == 1) return b;
+  apply_pass_fx<D, NV, NI, NO, 1>(b, a, M, tid, nth);
+  sync();
+  if (D == 2) return a;
+  apply_pass_fx<D, NV, NI, NO, 2>(a, b, M, tid, nth);
+  sync();
   return b;
 }
 
@@ -1239,8 +1292,8 @@ __global__ void __launch_bounds__(128, 8) k_correct_detect(Batch bt) {
   extern __shared__ double sm[];
   double* A = sm;                     // NV * BUF
   double* B = A + NV * BUF;           // NV * BUF
-  double* P1 = B + NV * BUF;          // Ns * n
-  double* lohi = P1 + Ns * n;         // 2 NV
+  FxOp* P1x = reinterpret_cast<FxOp*>(B + NV * BUF);   // Ns * n
+  double* lohi = reinterpret_cast<double*>(P1x + Ns * n);   // 2 NV
   double* mm = lohi + 2 * NV;         // 2 NV
   double* red = mm + 2 * NV;          // 128
   double* cw = red + 128;             // 2 D n: [k][side][a] dt/dx_k phi_side(a) / w_a
@@ -1248,9 +1301,10 @@ __global__ void __launch_bounds__(128, 8) k_correct_detect(Batch bt) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const Ops* o = bt.pps[0]->ops;
   for (int i = tid; i < Ns * n; i += nth) {
-    P1[i] = o->P1[i];
+    P1x[i] = o->P1x[i];
     P1f[i] = (float)o->P1[i];
   }
+  const FxMat P1m = {P1x, o->gP1, o->P1};
   __syncthreads();
   for (long long g = blockIdx.x; g < bt.pre[bt.n]; g += gridDim.x) {
     const int sidx = batch_state(bt, g);
@@ -1325,7 +1379,7 @@ __global__ void __launch_bounds__(128, 8) k_correct_detect(Batch bt) {
       }
       vs = A;
     } else {
-      vs = apply_ct<D, NV, n, Ns>(A, B, P1, tid, nth);
+      vs = apply_fx<D, NV, n, Ns>(A, B, P1m, tid, nth);
       if (vkeep)
         for (int e = tid; e < NV * NSD; e += nth) vkeep[e] = vs[e];
     }
@@ -1463,8 +1517,8 @@ __global__ void __launch_bounds__(32 * CD_WARPS) k_correct_detect_w(Batch bt) {
   using LY = CdLayout<D, N>;
   constexpr int n = DM::n, NV = DM::NV, ND = DM::ND, NF = DM::NF, Ns = DM::Ns, NSD = DM::NSD;
   extern __shared__ double sm[];
-  double* P1 = sm;
-  float* P1f = reinterpret_cast<float*>(P1 + Ns * n);
+  FxOp* P1x = reinterpret_cast<FxOp*>(sm);
+  float* P1f = reinterpret_cast<float*>(P1x + Ns * n);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double* A = sm + LY::OPS_DBL + w * LY::WARP_DBL;
   double* B = A + LY::A_DBL;
@@ -1472,9 +1526,10 @@ __global__ void __launch_bounds__(32 * CD_WARPS) k_correct_detect_w(Batch bt) {
   double* lohi = cw + LY::CW_DBL;
   const Ops* o = bt.pps[0]->ops;
   for (int i = threadIdx.x; i < Ns * n; i += 32 * CD_WARPS) {
-    P1[i] = o->P1[i];
+    P1x[i] = o->P1x[i];
     P1f[i] = (float)o->P1[i];
   }
+  const FxMat P1m = {P1x, o->gP1, o->P1};
   __syncthreads();
   const long long total = bt.pre[bt.n];
   for (long long g = (long long)blockIdx.x * CD_WARPS + w; g < total;
@@ -1550,7 +1605,7 @@ __global__ void __launch_bounds__(32 * CD_WARPS) k_correct_detect_w(Batch bt) {
       }
       vs = A;
     } else {
-      vs = apply_ct_warp<D, NV, n, Ns, double>(A, B, P1, lane);
+      vs = apply_fx<D, NV, n, Ns, true>(A, B, P1m, lane, 32);
       if (vkeep)
         for (int e = lane; e < NV * NSD; e += 32) vkeep[e] = vs[e];
     }

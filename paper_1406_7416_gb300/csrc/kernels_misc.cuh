@@ -17,16 +17,17 @@ __global__ void __launch_bounds__(128) k_load_detect(Params p, const double* __r
   extern __shared__ double sm[];
   double* A = sm;
   double* B = A + NV * NSD;
-  double* P1 = B + NV * NSD;
-  double* R1 = P1 + Ns * n;
-  double* lohi = R1 + n * Ns;
+  FxOp* P1x = reinterpret_cast<FxOp*>(B + NV * NSD);
+  FxOp* R1x = P1x + Ns * n;
+  double* lohi = reinterpret_cast<double*>(R1x + n * Ns);
   double* mm = lohi + 2 * NV;
   double* red = mm + 2 * NV;
   const int tid = threadIdx.x, nth = blockDim.x;
   for (int i = tid; i < Ns * n; i += nth) {
-    P1[i] = p.ops->P1[i];
-    R1[i] = p.ops->R1[i];
+    P1x[i] = p.ops->P1x[i];
+    R1x[i] = p.ops->R1x[i];
   }
+  const FxMat P1m = {P1x, p.ops->gP1, p.ops->P1}, R1m = {R1x, p.ops->gR1, p.ops->R1};
   __shared__ int s_slot;
   const int cur = p.cur;
   for (long long cell = blockIdx.x; cell < p.geo.cells; cell += gridDim.x) {
@@ -36,7 +37,7 @@ __global__ void __launch_bounds__(128) k_load_detect(Params p, const double* __r
     __syncthreads();
     for (int e = tid; e < NV * ND; e += nth) A[e] = U[e];
     __syncthreads();
-    double* vs = apply_ct<D, NV, n, Ns>(A, B, P1, tid, nth);
+    double* vs = apply_fx<D, NV, n, Ns>(A, B, P1m, tid, nth);
     if (exact) dmp_interval<D>(p, cmm_ex, ijk, lohi);
     __syncthreads();
     double lam;
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(128) k_load_detect(Params p, const double* __r
     }
     __syncthreads();
     check_subcells<D>(A, NSD, nullptr, p.gamma, mm, &lam, red);
-    double* u = apply_ct<D, NV, Ns, n>(A, B, R1, tid, nth);
+    double* u = apply_fx<D, NV, Ns, n>(A, B, R1m, tid, nth);
     for (int e = tid; e < NV * ND; e += nth) U[e] = u[e];
     if (tid == 0) {
       p.b.beta[cur][cell] = 1;
@@ -98,11 +99,12 @@ __global__ void __launch_bounds__(128) k_lambda(Params p) {
   extern __shared__ double sm[];
   double* A = sm;
   double* B = A + NV * NSD;
-  double* P1 = B + NV * NSD;
-  double* mm = P1 + Ns * n;
+  FxOp* P1x = reinterpret_cast<FxOp*>(B + NV * NSD);
+  double* mm = reinterpret_cast<double*>(P1x + Ns * n);
   double* red = mm + 2 * NV;
   const int tid = threadIdx.x, nth = blockDim.x;
-  for (int i = tid; i < Ns * n; i += nth) P1[i] = p.ops->P1[i];
+  for (int i = tid; i < Ns * n; i += nth) P1x[i] = p.ops->P1x[i];
+  const FxMat P1m = {P1x, p.ops->gP1, p.ops->P1};
   const int cur = p.cur;
   for (long long cell = blockIdx.x; cell < p.geo.cells; cell += gridDim.x) {
     __syncthreads();
@@ -116,7 +118,7 @@ __global__ void __launch_bounds__(128) k_lambda(Params p) {
       const double* U = p.b.U[cur] + cell * (NV * ND);
       for (int e = tid; e < NV * ND; e += nth) A[e] = U[e];
       __syncthreads();
-      vs = apply_ct<D, NV, n, Ns>(A, B, P1, tid, nth);
+      vs = apply_fx<D, NV, n, Ns>(A, B, P1m, tid, nth);
     }
     double lam;
     check_subcells<D>(vs, NSD, nullptr, p.gamma, mm, &lam, red);
@@ -152,12 +154,13 @@ __global__ void __launch_bounds__(128) k_load_full(Params p, const uint8_t* __re
   extern __shared__ double sm[];
   double* A = sm;
   double* B = A + NV * NSD;
-  double* P1 = B + NV * NSD;
-  double* mm = P1 + Ns * n;
+  FxOp* P1x = reinterpret_cast<FxOp*>(B + NV * NSD);
+  double* mm = reinterpret_cast<double*>(P1x + Ns * n);
   double* red = mm + 2 * NV;
   __shared__ int s_slot;
   const int tid = threadIdx.x, nth = blockDim.x;
-  for (int i = tid; i < Ns * n; i += nth) P1[i] = p.ops->P1[i];
+  for (int i = tid; i < Ns * n; i += nth) P1x[i] = p.ops->P1x[i];
+  const FxMat P1m = {P1x, p.ops->gP1, p.ops->P1};
   const int cur = p.cur;
   for (long long cell = blockIdx.x; cell < p.geo.cells; cell += gridDim.x) {
     __syncthreads();
@@ -195,7 +198,7 @@ __global__ void __launch_bounds__(128) k_load_full(Params p, const uint8_t* __re
         p.b.slot[cur][cell] = -1;
       }
       __syncthreads();
-      vs = apply_ct<D, NV, n, Ns>(A, B, P1, tid, nth);
+      vs = apply_fx<D, NV, n, Ns>(A, B, P1m, tid, nth);
     }
     double lam;
     check_subcells<D>(vs, NSD, nullptr, p.gamma, mm, &lam, red);

@@ -123,6 +123,25 @@ void basis_ops(int N, ld* xi, ld* w, ld* D, ld* Kt, ld* phi0, ld* phi1) {
     for (int j = 0; j < n; ++j) Kt[m * n + j] = K1[m * n + j] * w[j];
 }
 
+// Fixed-point form of a rows x cols operator (fixed.cuh: fx_scale, fx_op).
+int fixed_point(const double* M, int rows, int cols, FxOp* out) {
+  double s = 0.0;
+  for (int a = 0; a < rows; ++a) {
+    double r = 0.0;
+    for (int j = 0; j < cols; ++j) r += fabs(M[a * cols + j]);
+    s = r > s ? r : s;
+  }
+  int e;
+  frexp(s, &e);               // s < 2^e
+  const int g = e + 1;
+  for (int i = 0; i < rows * cols; ++i) {
+    const long long v = (long long)nearbyint(ldexp(M[i], 63 - g));
+    out[i].l = (int)(unsigned)(unsigned long long)v;
+    out[i].h = (int)((v - out[i].l) >> 32);
+  }
+  return g;
+}
+
 }  // namespace
 
 void build_ops(int N, Ops* o) {
@@ -182,6 +201,8 @@ void build_ops(int N, Ops* o) {
       o->P1[s * n + a] = (double)P1[s * n + a];
       o->Mt[a * Ns + s] = (double)(P1[s * n + a] / (Ns * w[a]));
     }
+  o->gP1 = fixed_point(o->P1, Ns, n, o->P1x);
+  o->gR1 = fixed_point(o->R1, n, Ns, o->R1x);
   // composite rule of the initial projection: Ns subintervals x (N+2) points
   {
     ld xq[MAXN + 1], wq[MAXN + 1];
