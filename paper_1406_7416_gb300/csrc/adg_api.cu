@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "adg_internal.h"
+#include "fork.h"
 
 using namespace adg;
 
@@ -455,12 +456,16 @@ int collect_phases(adg_state* st, int k) {
   return ADG_OK;
 }
 
-// Whether the state's predictor runs the split final stage (mixed precision
-// with no FP64 sweep) at a degree the warp-per-cell kernel covers.
-bool split_capable(const adg_state* st) {
+// Whether the state's predictor leaves split traces (mixed precision with no
+// FP64 sweep; kernels_dg.cuh: split_traces).
+bool split_traces_of(const adg_state* st) {
   const int f64 = st->fp64_sweeps < st->iters ? st->fp64_sweeps : st->iters;
-  return st->prec == ADG_PREC_MIXED_FP32 && f64 == 0 && st->iters > 0 &&
-         !(st->dim == 2 && st->N >= 6);
+  return st->prec == ADG_PREC_MIXED_FP32 && f64 == 0 && st->iters > 0;
+}
+
+// The same at a degree the warp-per-cell kernel covers.
+bool split_capable(const adg_state* st) {
+  return split_traces_of(st) && !(st->dim == 2 && st->N >= 6);
 }
 
 // Predictor shapes that apply to the state (PRED_*).
@@ -514,6 +519,8 @@ StepLaunch single_launch(adg_state* st) {
   sl.sub_f32 = st->sub_f32;
   sl.sub_reg = st->sub_reg;
   sl.flux = st->flux;
+  for (int k = 0; k < st->dim; ++k)
+    if (split_traces_of(st) && st->geo.periodic[k]) sl.split_periodic |= 1 << k;
   sl.total_cells = st->geo.cells;
   for (int k = 0; k < st->dim; ++k) {
     long long faces = 1;
@@ -656,7 +663,15 @@ int capture_step_graph(adg_state* st, StepLaunch* sls, adg_state* const* reps, i
     return fail(st, ADG_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
   }
   int rc = ADG_OK;
-  for (int i = 0; i < count && rc == ADG_OK; ++i) rc = enqueue_step(reps[i], sls[i], cap);
+  // the groups of a batch step different states: side by side
+  Fork fork(cap);
+  for (int i = 0; i < count && rc == ADG_OK; ++i) {
+    rc = enqueue_step(reps[i], sls[i], cap);
+    if (rc == ADG_OK && count > 1 && (e = fork.branch()) != cudaSuccess)
+      rc = fail(st, ADG_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
+  }
+  if (rc == ADG_OK && count > 1 && (e = fork.join()) != cudaSuccess)
+    rc = fail(st, ADG_ERR_CUDA, std::string("capture: ") + cudaGetErrorString(e));
   cudaGraph_t captured = nullptr;
   e = cudaStreamEndCapture(cap, &captured);
   if (rc || e != cudaSuccess) {
@@ -910,6 +925,7 @@ int adg_batch_create(adg_state* const* states, int count, void* stream, adg_batc
       pc[q + 1] = pc[q] + one.total_cells;
       for (int k = 0; k < 3; ++k) pf[k][q + 1] = pf[k][q] + one.total_faces[k];
       sum_chunk += st->chunk;
+      sl.split_periodic = q == 0 ? one.split_periodic : sl.split_periodic & one.split_periodic;
       if (st->cascade) sl.cascade = 1;
       const int passes = (st->cap + st->chunk - 1) / st->chunk;
       if (passes > max_passes) max_passes = passes;

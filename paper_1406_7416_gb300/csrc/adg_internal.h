@@ -182,6 +182,7 @@ struct StepLaunch {
   int sub_f32;                  // mixed precision: WENO3 reconstruction and sub-face fluxes in FP32
   int sub_reg;                 // the FP32 subcell predictor with a subcell in one warp's registers
   int flux;                    // numerical flux of the launch's states (ADG_FLUX_*)
+  int split_periodic;          // bit k: every state leaves split traces and is periodic along axis k
   int pred;                    // predictor launch shape (PRED_*)
   long long total_cells;
   long long total_faces[3];

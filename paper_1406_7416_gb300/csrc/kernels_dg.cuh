@@ -972,37 +972,25 @@ __device__ __forceinline__ void face_split_rusanov(const double* bL, const doubl
            0.5 * ((uR[v] - uL[v]) * Sd + widen_f32(sumJ[v]));
 }
 
-// One thread per (face, tangential node): the Rusanov (or Osher-type) flux at
-// each time node, weighted by the time rule.  At a domain boundary the missing
-// side is the ghost state of the face's kind (boundary_ghost).
+// One face node (a face normal to axis k, its tangential node ts) of a state:
+// the trace blocks on both sides and which sides are inside the domain.
 template <int D, int N>
-__global__ void __launch_bounds__(256, 2) k_faceflux(Batch bt, int k) {
+struct FaceNode {
   using DM = Dims<D, N>;
-  constexpr int n = DM::n, NV = DM::NV, NF = DM::NF, NT = DM::NT;
-  for (long long eg = blockIdx.x * (long long)blockDim.x + threadIdx.x; eg < bt.pre[bt.n];
-       eg += (long long)gridDim.x * blockDim.x) {
-    const int sidx = batch_state(bt, eg);
-    const Params& p = *bt.pps[sidx];
-    if (!(*p.b.dt > 0.0)) continue;
-    const long long e = eg - bt.pre[sidx];
+  int ijk[3];                // the face's index along k, its cell's along the others
+  int ts;
+  long long face;
+  bool hasL, hasR;
+  const double *trL, *trR;   // (a missing side takes the other's)
+
+  __device__ __forceinline__ FaceNode(const Params& p, int k, const int* at, int tsn) : ts(tsn) {
+    constexpr int n = DM::n, NV = DM::NV, NT = DM::NT;
     const Geo& g = p.geo;
-    const double* w = p.ops->w;
-    double* G = p.b.G[k];
-    const long long face = e / NF;
-    const int ts = (int)(e - face * NF);
-    int ijk[3] = {0, 0, 0};
-    long long r = face;
-#pragma unroll
-    for (int j = 0; j < D; ++j) {
-      const int ext = (j == k) ? g.n[j] + 1 : g.n[j];
-      ijk[j] = (int)(r % ext);
-      r /= ext;
-    }
-    const int f = ijk[k];
     int L[3], R[3];
 #pragma unroll
-    for (int j = 0; j < D; ++j) L[j] = R[j] = ijk[j];
-    bool hasL = true, hasR = true;
+    for (int j = 0; j < 3; ++j) L[j] = R[j] = ijk[j] = at[j];
+    const int f = ijk[k];
+    hasL = hasR = true;
     if (f == 0) {
       if (g.periodic[k]) L[k] = g.n[k] - 1; else hasL = false;
     } else {
@@ -1011,52 +999,195 @@ __global__ void __launch_bounds__(256, 2) k_faceflux(Batch bt, int k) {
     if (f == g.n[k]) {
       if (g.periodic[k]) R[k] = 0; else hasR = false;
     }
+    face = face_index<D>(g, ijk, k, f);
     const size_t csz = (size_t)D * 2 * NV * NT;
-    const double* trL = hasL ? p.b.trace + cell_index<D>(L, g) * csz + ((size_t)k * 2 + 1) * NV * NT
-                             : nullptr;
-    const double* trR = hasR ? p.b.trace + cell_index<D>(R, g) * csz + ((size_t)k * 2 + 0) * NV * NT
-                             : nullptr;
+    trL = hasL ? p.b.trace + cell_index<D>(L, g) * csz + ((size_t)k * 2 + 1) * NV * NT : nullptr;
+    trR = hasR ? p.b.trace + cell_index<D>(R, g) * csz + ((size_t)k * 2 + 0) * NV * NT : nullptr;
     if (!hasL) trL = trR;
     if (!hasR) trR = trL;
-    const bool split = split_traces(p);
-    double acc[NV];
-    if (split && hasL && hasR && p.flux == ADG_FLUX_RUSANOV) {
-      face_split_rusanov<D, n>(trL, trR, ts, k, p.gamma, p.ops->wf, p.b.coef_f[7], p.b.coef_f[6], acc);
+    (void)n;
+  }
+  __device__ __forceinline__ bool inside() const { return hasL && hasR; }
+
+  // The numerical flux at time node m; at a domain boundary the missing side
+  // is the ghost state of the face's kind (boundary_ghost).
+  template <bool OSHER>
+  __device__ __forceinline__ void flux(const Params& p, int k, int m, bool split, double* Gm) const {
+    constexpr int n = DM::n, NV = DM::NV;
+    const Geo& g = p.geo;
+    double QL[NV], QR[NV];
+    load_trace<D, n>(trL, ts, m, split, QL);
+    load_trace<D, n>(trR, ts, m, split, QR);
+    if (!hasL || !hasR) {
+      const int side = 2 * k + (hasL ? 1 : 0);
+      double pos = 0.0, t = 0.0;
+      if (g.bc[side] == ADG_BC_FRONT) {
+        // the node's coordinate along the front's axis, and its time
+        const int j = g.front_axis[side];
+        int a = 0, tt = ts;
 #pragma unroll
-      for (int v = 0; v < NV; ++v) G[(face * NV + v) * NF + ts] = acc[v];
-      continue;
-    }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = 0.0;
-    for (int m = 0; m < n; ++m) {
-      double QL[NV], QR[NV], Gm[NV];
-      load_trace<D, n>(trL, ts, m, split, QL);
-      load_trace<D, n>(trR, ts, m, split, QR);
-      if (!hasL || !hasR) {
-        const int face = 2 * k + (hasL ? 1 : 0);
-        double pos = 0.0, t = 0.0;
-        if (g.bc[face] == ADG_BC_FRONT) {
-          // the node's coordinate along the front's axis, and its time
-          const int j = g.front_axis[face];
-          int a = 0, tt = ts;
-#pragma unroll
-          for (int jj = 0; jj < D; ++jj)
-            if (jj != k) {
-              if (jj == j) a = tt % n;
-              tt /= n;
-            }
-          pos = g.x0[j] + (ijk[j] + p.ops->xi[a]) * g.dx[j];
-          t = *p.b.tstart + p.ops->xi[m] * *p.b.dt;
-        }
-        if (!hasL) boundary_ghost<D>(g, face, QR, QL, pos, t);
-        else boundary_ghost<D>(g, face, QL, QR, pos, t);
+        for (int jj = 0; jj < D; ++jj)
+          if (jj != k) {
+            if (jj == j) a = tt % n;
+            tt /= n;
+          }
+        pos = g.x0[j] + (ijk[j] + p.ops->xi[a]) * g.dx[j];
+        t = *p.b.tstart + p.ops->xi[m] * *p.b.dt;
       }
-      face_flux<D>(p.flux, QL, QR, k, p.gamma, Gm, p.prec == ADG_PREC_MIXED_FP32);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) acc[v] += w[m] * Gm[v];
+      if (!hasL) boundary_ghost<D>(g, side, QR, QL, pos, t);
+      else boundary_ghost<D>(g, side, QL, QR, pos, t);
     }
+    face_flux<D>(OSHER ? ADG_FLUX_OSHER : ADG_FLUX_RUSANOV, QL, QR, k, p.gamma, Gm,
+                 p.prec == ADG_PREC_MIXED_FP32);
+  }
+};
+
+// Time-averaged numerical flux at every face node normal to axis k.  Past the
+// first `wide_blocks` blocks, one thread takes a node inside the domain and
+// steps through its time nodes.  The first blocks take n lanes per node, one
+// per time node, and add the n fluxes in order from one lane to the next (the
+// same operations: the same bits): the nodes on the domain's boundary, whose
+// ghost states and FP64 fluxes at n time nodes in a row kept one warp busy long
+// after the other faces were done, or with `wide` (few nodes: waiting for one
+// thread's n fluxes is then the whole kernel) every node that is not a split
+// Rusanov one, whose time nodes are FP32.
+// Measured (GB300), face fluxes per step with the axes side by side: 32^2 N = 3
+// mixed, transmissive, 49 -> 17 us; 350 x 100 N = 5 mixed (inflow, wall, fronts)
+// 178 -> 74 us; 64^3 N = 3 mixed 2.63 -> 1.92 ms; 256^2 N = 5 FP64 0.77 -> 0.66.
+//
+// KIND: FACE_OSHER, FACE_RUSANOV, or FACE_LEAN for launches whose nodes are all
+// split Rusanov ones inside the domain (mixed precision, periodic axis): without
+// the general path's registers more warps hide that path's load latency.
+// K: the axis at compile time (-1: taken from `axis`; the Osher-type flux only),
+// so that the states' and fluxes' k-th components are registers and not an
+// indexed array in local memory.  512^2 N = 5 mixed (lean): 0.71 -> 0.38 ms per
+// step at three blocks per SM, 0.35 at four, 0.51 at two.
+enum FaceKind { FACE_RUSANOV, FACE_OSHER, FACE_LEAN };
+
+template <int D, int N, int KIND, int K>
+__global__ void __launch_bounds__(256, KIND == FACE_LEAN ? 4 : (D == 2 && N >= 6 ? 2 : 3))
+    k_faceflux(Batch bt, int axis, int wide_blocks, int wide) {
+  const int k = K >= 0 ? K : axis;
+  using DM = Dims<D, N>;
+  constexpr int n = DM::n, NV = DM::NV, NF = DM::NF;
+  if ((int)blockIdx.x >= wide_blocks) {
+    for (long long eg = (long long)(blockIdx.x - wide_blocks) * blockDim.x + threadIdx.x; eg < bt.pre[bt.n];
+         eg += (long long)(gridDim.x - wide_blocks) * blockDim.x) {
+      const int sidx = batch_state(bt, eg);
+      const Params& p = *bt.pps[sidx];
+      if (!(*p.b.dt > 0.0)) continue;
+      const long long e = eg - bt.pre[sidx];
+      const Geo& g = p.geo;
+      const long long face = e / NF;
+      int ijk[3] = {0, 0, 0};
+      long long r = face;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) G[(face * NV + v) * NF + ts] = acc[v];
+      for (int j = 0; j < D; ++j) {
+        const int ext = (j == k) ? g.n[j] + 1 : g.n[j];
+        ijk[j] = (int)(r % ext);
+        r /= ext;
+      }
+      if (KIND != FACE_LEAN && !g.periodic[k] && (ijk[k] == 0 || ijk[k] == g.n[k])) continue;
+      const bool split = KIND == FACE_LEAN || split_traces(p);
+      const bool fp32 = split && KIND != FACE_OSHER;
+      if (KIND != FACE_LEAN && wide && !fp32) continue;
+      const FaceNode<D, N> fn(p, k, ijk, (int)(e - face * NF));
+      double* G = p.b.G[k] + face * (NV * NF) + fn.ts;
+      double acc[NV];
+      if (KIND == FACE_LEAN || fp32) {
+        face_split_rusanov<D, n>(fn.trL, fn.trR, fn.ts, k, p.gamma, p.ops->wf, p.b.coef_f[7],
+                                 p.b.coef_f[6], acc);
+      } else {
+        const double* w = p.ops->w;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+        for (int m = 0; m < n; ++m) {
+          double Gm[NV];
+          fn.template flux<KIND == FACE_OSHER>(p, k, m, split, Gm);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) acc[v] += w[m] * Gm[v];
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) G[v * NF] = acc[v];
+    }
+    return;
+  }
+  if constexpr (KIND != FACE_LEAN) {
+  constexpr int GPW = 32 / n;                            // nodes per warp
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int grp = lane / n < GPW ? lane / n : GPW - 1;   // (idle lanes repeat the last node's)
+  const int m = lane / n < GPW ? lane - grp * n : n - 1;
+  const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const long long stride = (long long)wide_blocks * (blockDim.x >> 5) * GPW;
+  for (long long q0 = warp * GPW;; q0 += stride) {       // (uniform over the warp)
+    // node q: the q-th of all (wide), or of the boundary nodes of state after state
+    long long q = q0 + grp;
+    const Params* pp = nullptr;
+    int ijk[3] = {0, 0, 0}, ts = 0;
+    if (wide) {
+      if (q0 >= bt.pre[bt.n]) break;
+      if (q < bt.pre[bt.n]) {
+        const int s = batch_state(bt, q);
+        pp = bt.pps[s];
+        q -= bt.pre[s];
+        ts = (int)(q % NF);
+        q /= NF;
+#pragma unroll
+        for (int j = 0; j < D; ++j) {
+          const int ext = (j == k) ? pp->geo.n[j] + 1 : pp->geo.n[j];
+          ijk[j] = (int)(q % ext);
+          q /= ext;
+        }
+      }
+    } else {
+      long long left = q;
+      for (int s = 0; s < bt.n && !pp; ++s) {
+        const Geo& g = bt.pps[s]->geo;
+        if (g.periodic[k]) continue;
+        const long long cnt = 2 * (g.cells / g.n[k]) * NF;
+        if (left < cnt) {
+          pp = bt.pps[s];
+          ts = (int)(left % NF);
+          left /= NF;
+          ijk[k] = (left & 1) ? g.n[k] : 0;
+          left >>= 1;
+#pragma unroll
+          for (int j = 0; j < D; ++j)
+            if (j != k) {
+              ijk[j] = (int)(left % g.n[j]);
+              left /= g.n[j];
+            }
+        } else {
+          left -= cnt;
+        }
+      }
+      if (!__any_sync(FULL, pp != nullptr)) break;
+    }
+    double Gm[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Gm[v] = 0.0;
+    double* G = nullptr;
+    if (pp && *pp->b.dt > 0.0) {
+      const Params& p = *pp;
+      const FaceNode<D, N> fn(p, k, ijk, ts);
+      const bool split = split_traces(p);
+      if (!fn.inside() || !split || KIND == FACE_OSHER) {
+        fn.template flux<KIND == FACE_OSHER>(p, k, m, split, Gm);
+        G = p.b.G[k] + fn.face * (NV * NF) + ts;
+      }
+    }
+    const double* w = bt.pps[0]->ops->w;                 // (every state of a batch has degree N)
+    __syncwarp();
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      double acc = 0.0;
+#pragma unroll
+      for (int i = 0; i < n; ++i) acc += w[i] * __shfl_sync(FULL, Gm[v], grp * n + i);
+      if (G && m == v % n && lane < GPW * n) G[v * NF] = acc;
+    }
+  }
   }
 }
 

@@ -1,6 +1,7 @@
 // Launch configuration of every kernel for one (dimension, degree).
 #pragma once
 
+#include "fork.h"
 #include "kernels_misc.cuh"
 #include "kernels_pred.cuh"
 
@@ -173,6 +174,14 @@ struct Launch {
     return 64;
   }
 
+  template <int K>
+  static void launch_face(const Batch& faces, const StepLaunch& sl, int mb, int wb, bool wide, cudaStream_t s) {
+    if (sl.split_periodic >> K & 1)
+      k_faceflux<D, N, FACE_LEAN, K><<<mb, 256, 0, s>>>(faces, K, 0, 0);
+    else
+      k_faceflux<D, N, FACE_RUSANOV, K><<<mb + wb, 256, 0, s>>>(faces, K, wb, wide ? 1 : 0);
+  }
+
   static cudaError_t step_dg(const StepLaunch& sl, cudaStream_t s) {
     cudaError_t e;
     cudaEvent_t* ev = sl.ev;
@@ -182,9 +191,29 @@ struct Launch {
     mark(ev, PHASE_PREDICTOR, s);
     if ((e = launch_predictor(sl, s)) != cudaSuccess) return e;
     mark(ev, PHASE_FACEFLUX, s);
-    for (int k = 0; k < D; ++k) {
-      const Batch faces{sl.pps, sl.n, sl.pre_faces[k]};
-      k_faceflux<D, N><<<grid_for(sl.total_faces[k], 256), 256, 0, s>>>(faces, k);
+    {
+      Fork fork(s);
+      for (int k = 0; k < D; ++k) {
+        const Batch faces{sl.pps, sl.n, sl.pre_faces[k]};
+        // n lanes per node: every node up to eight warps of time nodes per SM
+        // (there the FP64 fluxes themselves take less than one thread's n in a
+        // row; at 67 x 53, N = 6, 36 warps per SM, it was 11% slower), else the
+        // boundary's, of the order of cells / n_k, on at most one block per SM
+        constexpr int per_block = 8 * (32 / n);
+        const bool wide = sl.total_faces[k] * n <= (long long)kNumSM * 256;
+        const int wb = grid_for(sl.total_faces[k], per_block, wide ? kNumSM * 2 : kNumSM);
+        const int mb = grid_for(sl.total_faces[k], 256);
+        if (sl.flux == ADG_FLUX_OSHER)
+          k_faceflux<D, N, FACE_OSHER, -1><<<mb + wb, 256, 0, s>>>(faces, k, wb, wide ? 1 : 0);
+        else if (k == 0)
+          launch_face<0>(faces, sl, mb, wb, wide, s);
+        else if (k == 1)
+          launch_face<1>(faces, sl, mb, wb, wide, s);
+        else
+          launch_face<D - 1>(faces, sl, mb, wb, wide, s);
+        if ((e = fork.branch()) != cudaSuccess) return e;
+      }
+      if ((e = fork.join()) != cudaSuccess) return e;
     }
     mark(ev, PHASE_CORRECT, s);
     if constexpr (D == 2) {
@@ -220,17 +249,24 @@ struct Launch {
     static const int gw = persistent_grid(k_lim_flux_d<D, N, K, OSHER>, 128, 0, 1LL << 40);
     k_lim_flux_d<D, N, K, OSHER><<<(int)(want < gw ? want : gw), 128, 0, s>>>(lim, pass);
   }
-  static void launch_flux_d(const Batch& lim, int pass, long long ch, int flux, cudaStream_t s) {
+  template <bool OSHER>
+  static cudaError_t launch_flux_axes(const Batch& lim, int pass, long long ch, cudaStream_t s) {
     const long long want = (ch * (Ns + 1) * DM::NSF / FluxPoints<D>::FACES + 4) / 4;
-    if (flux == ADG_FLUX_OSHER) {
-      launch_flux_axis<0, true>(lim, pass, want, s);
-      launch_flux_axis<1, true>(lim, pass, want, s);
-      if constexpr (D == 3) launch_flux_axis<2, true>(lim, pass, want, s);
-    } else {
-      launch_flux_axis<0, false>(lim, pass, want, s);
-      launch_flux_axis<1, false>(lim, pass, want, s);
-      if constexpr (D == 3) launch_flux_axis<2, false>(lim, pass, want, s);
+    cudaError_t e;
+    Fork fork(s);
+    launch_flux_axis<0, OSHER>(lim, pass, want, s);
+    if ((e = fork.branch()) != cudaSuccess) return e;
+    launch_flux_axis<1, OSHER>(lim, pass, want, s);
+    if ((e = fork.branch()) != cudaSuccess) return e;
+    if constexpr (D == 3) {
+      launch_flux_axis<2, OSHER>(lim, pass, want, s);
+      if ((e = fork.branch()) != cudaSuccess) return e;
     }
+    return fork.join();
+  }
+  static cudaError_t launch_flux_d(const Batch& lim, int pass, long long ch, int flux, cudaStream_t s) {
+    return flux == ADG_FLUX_OSHER ? launch_flux_axes<true>(lim, pass, ch, s)
+                                  : launch_flux_axes<false>(lim, pass, ch, s);
   }
 
   // One limiter pass (pass < 0: the pass of the device-sized loop).
@@ -304,8 +340,11 @@ struct Launch {
         const long long want = ((ch * (Ns + 1) * DM::NSF + 2) / 3 + 7) / 8;
         static const int g0 = persistent_grid(k_lim_flux_t2<N, 0>, 256, 0, 1LL << 40);
         static const int g1 = persistent_grid(k_lim_flux_t2<N, 1>, 256, 0, 1LL << 40);
+        Fork fork(s);
         k_lim_flux_t2<N, 0><<<(int)(want < g0 ? want : g0), 256, 0, s>>>(lim, pass);
+        if ((e = fork.branch()) != cudaSuccess) return e;
         k_lim_flux_t2<N, 1><<<(int)(want < g1 ? want : g1), 256, 0, s>>>(lim, pass);
+        if ((e = fork.branch()) != cudaSuccess || (e = fork.join()) != cudaSuccess) return e;
       }
     } else if (traces) {
       if constexpr (D == 3) {
@@ -314,9 +353,13 @@ struct Launch {
         static const int g0 = persistent_grid(k_lim_flux_t<N, 0>, 256, 0, 1LL << 40);
         static const int g1 = persistent_grid(k_lim_flux_t<N, 1>, 256, 0, 1LL << 40);
         static const int g2 = persistent_grid(k_lim_flux_t<N, 2>, 256, 0, 1LL << 40);
+        Fork fork(s);
         k_lim_flux_t<N, 0><<<(int)(want < g0 ? want : g0), 256, 0, s>>>(lim, pass);
+        if ((e = fork.branch()) != cudaSuccess) return e;
         k_lim_flux_t<N, 1><<<(int)(want < g1 ? want : g1), 256, 0, s>>>(lim, pass);
+        if ((e = fork.branch()) != cudaSuccess) return e;
         k_lim_flux_t<N, 2><<<(int)(want < g2 ? want : g2), 256, 0, s>>>(lim, pass);
+        if ((e = fork.branch()) != cudaSuccess || (e = fork.join()) != cudaSuccess) return e;
       }
     } else if (sl.prec == ADG_PREC_MIXED_FP32 && sl.sub_f32 && sl.flux == ADG_FLUX_RUSANOV) {
       if (qf) {
@@ -333,7 +376,7 @@ struct Launch {
       k_lim_flux<D, N, 1, double, float><<<gf, 256, 0, s>>>(lim, pass);
       if (D == 3) k_lim_flux<D, N, (D == 3 ? 2 : 1), double, float><<<gf, 256, 0, s>>>(lim, pass);
     } else {
-      launch_flux_d(lim, pass, ch, sl.flux, s);
+      if ((e = launch_flux_d(lim, pass, ch, sl.flux, s)) != cudaSuccess) return e;
     }
     k_lim_update<D, N><<<(int)(ch < kNumSM * 8 ? ch : kNumSM * 8), 128, cell_smem(), s>>>(lim, pass);
     return cudaGetLastError();
@@ -369,6 +412,8 @@ struct Launch {
       for (int pass = 0; pass < sl.max_passes; ++pass)
         if ((e = lim_pass(sl, pass, s)) != cudaSuccess) return e;
     }
+    const size_t sf = fix_smem();
+    if ((e = set_smem(k_lim_fix<D, N>, sf)) != cudaSuccess) return e;
     if (sl.cascade) {
       // first-order layer after WENO3 (Sec. 6, Fig. algo2); both lists are
       // empty in most steps and the kernels then return at once
@@ -376,16 +421,25 @@ struct Launch {
       const size_t sfb = fallback_smem();
       if ((e = set_smem(k_lim_fallback<D, N>, sfb)) != cudaSuccess) return e;
       k_lim_fallback<D, N><<<kNumSM, 128, sfb, s>>>(Batch{sl.pps, sl.n, sl.pre_fb});
-      if ((e = launch_count_prefix(sl, sl.pre_refix, CNT_REFIX, s)) != cudaSuccess) return e;
       if ((e = set_smem(k_lim_refix<D, N>, su)) != cudaSuccess) return e;
+    }
+    // The fix of unlimited neighbours needs the first-order fluxes but not the
+    // rebalanced WENO3 cells (it writes unlimited cells, reads them and the edge
+    // fluxes): the two run side by side.  (A phase event between them keeps them
+    // in order.)
+    Fork fork(s);
+    if (sl.cascade) {
+      if ((e = launch_count_prefix(sl, sl.pre_refix, CNT_REFIX, s)) != cudaSuccess) return e;
       k_lim_refix<D, N><<<kNumSM, 128, su, s>>>(Batch{sl.pps, sl.n, sl.pre_refix});
+      if (!ev && (e = fork.branch()) != cudaSuccess) return e;
     }
     mark(ev, PHASE_FIX, s);
     if ((e = launch_fix_prefix(sl, s)) != cudaSuccess) return e;
-    const size_t sf = fix_smem();
-    if ((e = set_smem(k_lim_fix<D, N>, sf)) != cudaSuccess) return e;
     const Batch fix{sl.pps, sl.n, sl.pre_fix};
     k_lim_fix<D, N><<<kNumSM * 8, 128, sf, s>>>(fix);
+    if (!ev) {
+      if ((e = fork.branch()) != cudaSuccess || (e = fork.join()) != cudaSuccess) return e;
+    }
     mark(ev, PHASE_END, s);
     return cudaGetLastError();
   }

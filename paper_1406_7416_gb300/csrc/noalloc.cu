@@ -160,7 +160,8 @@ struct NoAlloc {
       k_lim_sweep<D, N, (D == 3 ? 2 : 1), double><<<grid_for(ch * DM::NV * DM::LD, 256), 256, 0, s>>>(lim, 0);
     const long long ncross = ch * (DM::NSD + 2 * D * DM::NSF);
     Launch<D, N>::template launch_predict_i<double>(lim, ncross, s);
-    Launch<D, N>::launch_flux_d(lim, 0, ch, ADG_FLUX_RUSANOV, s);
+    const cudaError_t ef = Launch<D, N>::launch_flux_d(lim, 0, ch, ADG_FLUX_RUSANOV, s);
+    if (ef != cudaSuccess) return ef;
     k_noalloc_write<D, N><<<grid_for(ch * DM::NV * DM::NSD, 256), 256, 0, s>>>(p, count, vnew, faces);
     return cudaGetLastError();
   }
