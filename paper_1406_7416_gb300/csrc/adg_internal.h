@@ -51,9 +51,9 @@ struct Ops {
   // averages, Wf[k][node * 3 + r] = sum_p E[node][p] C[k][p][r]
   float Cf[3][6];
   float Wf[3][9];
-  // P1 and R1 for the integer pipes (fixed.cuh), with their scale exponents
-  FxOp P1x[MAXNS * MAXN], R1x[MAXN * MAXNS];
-  int gP1, gR1;
+  // P1 for the integer pipes (fixed.cuh), with its scale exponent
+  FxOp P1x[MAXNS * MAXN];
+  int gP1;
 };
 
 // Builds the operator table of degree N (host, long double arithmetic).
@@ -621,13 +621,16 @@ __device__ __forceinline__ double wave_speed_f(const double* Q, double pe, float
 // ---------------------------------------------------------------------------
 // Grid helpers
 // ---------------------------------------------------------------------------
+// (32-bit divisions, a grid has less than 2^31 cells: a 64-bit one by a run-time
+// divisor is a call whose conversions run on the FP64 pipe)
 template <int D>
 __device__ __forceinline__ void cell_coords(long long c, const Geo& g, int* ijk) {
-  ijk[0] = (int)(c % g.n[0]);
-  long long r = c / g.n[0];
+  const unsigned u = (unsigned)c, n0 = (unsigned)g.n[0], r = u / n0;
+  ijk[0] = (int)(u - r * n0);
   if (D == 3) {
-    ijk[1] = (int)(r % g.n[1]);
-    ijk[2] = (int)(r / g.n[1]);
+    const unsigned n1 = (unsigned)g.n[1], z = r / n1;
+    ijk[1] = (int)(r - z * n1);
+    ijk[2] = (int)z;
   } else {
     ijk[1] = (int)r;
   }

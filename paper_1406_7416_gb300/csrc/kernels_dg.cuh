@@ -190,6 +190,8 @@ __device__ __forceinline__ void time_fx(const double* F, double* q, const double
 // its FMA, so the FP32 sweeps load only their data from shared memory.
 static __constant__ float c_Dmf[MAXN][MAXN * MAXN];
 static __constant__ float c_Ktf[MAXN][MAXN * MAXN];
+// the projection P of every degree
+static __constant__ float c_P1f[MAXN][MAXNS * MAXN];
 // the degree-2 subcell predictor's operators (3 nodes), likewise
 static __constant__ float c_D3f[9];
 static __constant__ float c_K3f[9];
@@ -427,21 +429,71 @@ __device__ __forceinline__ void apply_pass_ct(const T* __restrict__ in, T* __res
   }
 }
 
-template <int D, int NV, int NI, int NO, typename T>
-__device__ __forceinline__ T* apply_ct(T* a, T* b, const T* M, int tid, int nth) {
-  apply_pass_ct<D, NV, NI, NO, 0, T>(a, b, M, tid, nth);
+// One pass of the FP32 projection P of the step's change: one thread per line of
+// n nodes along axis K, its Ns outputs' operator entries from constant memory
+// (the sums in the order of apply_pass_ct).  One thread per output loaded 2 n
+// operands for n FMAs.  With it the detector's scan reads and updates the kept
+// averages itself (no copy of them in shared memory, one barrier fewer) and
+// reduces its extremes by warp_max_key: 5022 -> 3774 instructions per 2D N = 5
+// cell.  Measured (GB300), corrector and detector per step, mixed: 512^2 N = 5
+// 2.14 -> 1.86 ms, 200^2 N = 9 1.65 -> 1.35, 64^3 N = 3 10.1 -> 8.1.
+template <int D, int N, int K>
+__device__ __forceinline__ void project_pass_f(const float* in, float* out, int tid, int nth) {
+  constexpr int NV = D + 2, NI = N + 1, NO = 2 * N + 1;
+  constexpr int I0 = (0 < K) ? NO : NI, I1 = (D < 2) ? 1 : ((1 < K) ? NO : NI), I2 = (D < 3) ? 1 : NI;
+  constexpr int ISZ = I0 * I1 * I2, LINES = ISZ / NI, OSZ = LINES * NO;
+  constexpr int S = (K == 0) ? 1 : (K == 1 ? I0 : I0 * I1);       // stride along K, in and out
+  for (int e = tid; e < NV * LINES; e += nth) {
+    const int v = e / LINES, r = e - v * LINES;
+    const int lo = r % S, hi = r / S;
+    const float* src = in + v * ISZ + lo + hi * (S * NI);
+    float* dst = out + v * OSZ + lo + hi * (S * NO);
+    float x[NI];
+#pragma unroll
+    for (int j = 0; j < NI; ++j) x[j] = src[j * S];
+#pragma unroll
+    for (int a = 0; a < NO; ++a) {
+      float acc = 0.0f;
+#pragma unroll
+      for (int j = 0; j < NI; ++j) acc += c_P1f[N][a * NI + j] * x[j];
+      dst[a * S] = acc;
+    }
+  }
+}
+
+template <int D, int N, bool WARP>
+__device__ __forceinline__ const float* project_f(float* a, float* b, int tid, int nth) {
+  auto sync = [] {
+    if (WARP) __syncwarp();
+    else __syncthreads();
+  };
+  project_pass_f<D, N, 0>(a, b, tid, nth);
+  sync();
+  project_pass_f<D, N, 1>(b, a, tid, nth);
+  sync();
+  if (D == 2) return a;
+  project_pass_f<D, N, 2>(a, b, tid, nth);
+  sync();
+  return b;
+}
+
+// Tensor reconstruction R of one cell in FP64 (few cells: the FMA chain, whose
+// DOFs the FP32 subcell and predictor kernels round from).
+template <int D, int N>
+__device__ __forceinline__ double* reconstruct(double* a, double* b, const double* R1, int tid, int nth) {
+  constexpr int NV = D + 2, n = N + 1, Ns = 2 * N + 1;
+  apply_pass_ct<D, NV, Ns, n, 0, double>(a, b, R1, tid, nth);
   __syncthreads();
-  if (D == 1) return b;
-  apply_pass_ct<D, NV, NI, NO, 1, T>(b, a, M, tid, nth);
+  apply_pass_ct<D, NV, Ns, n, 1, double>(b, a, R1, tid, nth);
   __syncthreads();
   if (D == 2) return a;
-  apply_pass_ct<D, NV, NI, NO, 2, T>(a, b, M, tid, nth);
+  apply_pass_ct<D, NV, Ns, n, 2, double>(a, b, R1, tid, nth);
   __syncthreads();
   return b;
 }
 
-// The FP64 operator of a projection or reconstruction: its fixed-point entries
-// (shared memory) with their scale exponent, and its doubles.
+// The FP64 projection operator: its fixed-point entries (shared memory) with
+// their scale exponent, and its doubles.
 struct FxMat {
   const FxOp* x;
   int g;
@@ -474,8 +526,7 @@ __device__ __forceinline__ void apply_pass_fx(const double* in, double* out, con
   }
 }
 
-// Tensor projection / reconstruction in FP64 through two buffers, by a block
-// or (WARP) a warp.
+// Tensor projection in FP64 through two buffers, by a block or (WARP) a warp.
 template <int D, int NV, int NI, int NO, bool WARP = false>
 __device__ __forceinline__ double* apply_fx(double* a, double* b, const FxMat& M, int tid, int nth) {
   auto sync = [] {
@@ -1065,7 +1116,7 @@ struct FaceNode {
 enum FaceKind { FACE_RUSANOV, FACE_OSHER, FACE_LEAN };
 
 template <int D, int N, int KIND, int K>
-__global__ void __launch_bounds__(256, KIND == FACE_LEAN ? 4 : (D == 2 && N >= 6 ? 2 : 3))
+__global__ void __launch_bounds__(256, KIND == FACE_OSHER ? 2 : (KIND == FACE_LEAN ? 6 - D : (D == 2 && N >= 6 ? 2 : 3)))
     k_faceflux(Batch bt, int axis, int wide_blocks, int wide) {
   const int k = K >= 0 ? K : axis;
   using DM = Dims<D, N>;
@@ -1080,12 +1131,17 @@ __global__ void __launch_bounds__(256, KIND == FACE_LEAN ? 4 : (D == 2 && N >= 6
       const Geo& g = p.geo;
       const long long face = e / NF;
       int ijk[3] = {0, 0, 0};
-      long long r = face;
+      // (32-bit divisions as in cell_coords: faces along an axis < 2^32)
+      unsigned r = (unsigned)face;
 #pragma unroll
       for (int j = 0; j < D; ++j) {
-        const int ext = (j == k) ? g.n[j] + 1 : g.n[j];
-        ijk[j] = (int)(r % ext);
-        r /= ext;
+        if (j + 1 < D) {
+          const unsigned ext = (unsigned)((j == k) ? g.n[j] + 1 : g.n[j]), t = r / ext;
+          ijk[j] = (int)(r - t * ext);
+          r = t;
+        } else {
+          ijk[j] = (int)r;
+        }
       }
       if (KIND != FACE_LEAN && !g.periodic[k] && (ijk[k] == 0 || ijk[k] == g.n[k])) continue;
       const bool split = KIND == FACE_LEAN || split_traces(p);
@@ -1248,23 +1304,36 @@ __device__ __forceinline__ long long speed_key(double s) {
   return isnan_f64(s) ? LLONG_MAX : ord_key(s);
 }
 
+// Key of an interval's end for the test on keys, key(x) >= key(lo) && key(x) <=
+// key(hi): exactly the FP64 comparisons (a zero of either sign is the lower
+// zero below and the upper zero above; a NaN end fails every x but NaN, which
+// fails at the other end).  FP64 comparisons run on the FP64 pipe, once for
+// every warp here.
+__device__ __forceinline__ long long bound_key(double x, bool high) {
+  if (isnan_f64(x)) return high ? LLONG_MIN : LLONG_MAX;
+  const long long b = __double_as_longlong(x);
+  if ((b << 1) == 0) return high ? 0 : -1;
+  return ord_key(x);
+}
+
 // Detector bounds over the Voronoi neighbourhood (3^d block) from per-cell
 // min/max, then the relaxed DMP interval [m - delta, M + delta] (Eq. relax
-// with a relative floor).  Threads v < nvar write lohi[2v], lohi[2v+1].
+// with a relative floor).  Threads v < nvar write the keys of its ends
+// (bound_key), lohi[2v], lohi[2v+1].
 template <int D>
 __device__ __forceinline__ void dmp_interval_lane(const Params& p, const double* __restrict__ cmm,
-                                                  const int* ijk, double* lohi, int v);
+                                                  const int* ijk, long long* lohi, int v);
 
 template <int D>
 __device__ __forceinline__ void dmp_interval(const Params& p, const double* __restrict__ cmm,
-                                             const int* ijk, double* lohi) {
+                                             const int* ijk, long long* lohi) {
   if ((int)threadIdx.x < D + 2) dmp_interval_lane<D>(p, cmm, ijk, lohi, threadIdx.x);
 }
 
 // The interval of variable v (one thread per variable).
 template <int D>
 __device__ __forceinline__ void dmp_interval_lane(const Params& p, const double* __restrict__ cmm,
-                                                  const int* ijk, double* lohi, int v) {
+                                                  const int* ijk, long long* lohi, int v) {
   const int NV = D + 2;
   const Geo& g = p.geo;
   // min / max on order-preserving integer keys (the integer pipe), NaNs
@@ -1308,8 +1377,17 @@ __device__ __forceinline__ void dmp_interval_lane(const Params& p, const double*
   // (the same result; the FP64 pipe runs fmax)
   const double scale = max_nonneg(1.0, max_nonneg(fabs(mx), fabs(mn)));
   const double delta = max_nonneg(p.eps * (mx - mn), p.floor * scale);
-  lohi[2 * v] = mn - delta;
-  lohi[2 * v + 1] = mx + delta;
+  lohi[2 * v] = bound_key(mn - delta, false);
+  lohi[2 * v + 1] = bound_key(mx + delta, true);
+}
+
+// The largest of the warp's 64-bit keys, in every lane: the largest high words
+// by one 32-bit reduction, then the largest low word among the lanes that have
+// it (a shuffle tree of 64-bit maxima takes five times as many instructions).
+__device__ __forceinline__ long long warp_max_key(long long k) {
+  const int h = __reduce_max_sync(0xffffffffu, (int)(k >> 32));
+  const unsigned l = __reduce_max_sync(0xffffffffu, (int)(k >> 32) == h ? (unsigned)k : 0u);
+  return ((long long)h << 32) | l;
 }
 
 // Max-reduces K integer keys per thread over the block (blockDim a multiple of
@@ -1317,8 +1395,7 @@ __device__ __forceinline__ void dmp_interval_lane(const Params& p, const double*
 template <int K>
 __device__ __forceinline__ const long long* block_max_keys(long long* r, long long* red) {
 #pragma unroll
-  for (int j = 0; j < K; ++j)
-    for (int o = 16; o > 0; o >>= 1) r[j] = max(r[j], __shfl_xor_sync(0xffffffffu, r[j], o));
+  for (int j = 0; j < K; ++j) r[j] = warp_max_key(r[j]);
   const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   __syncthreads();
   if ((threadIdx.x & 31) == 0)
@@ -1334,29 +1411,27 @@ __device__ __forceinline__ const long long* block_max_keys(long long* r, long lo
   return red + nw * K;
 }
 
-// Checks the subcell data vs[v][s] of one cell.
+// Checks of the subcell data of one cell, value(v, s) (called once per variable
+// and subcell):
 //   PAD: rho > 0 and rho E - |m|^2 / 2 > 0 on every subcell (for rho > 0 the
 //        second test is p > 0 without a division; NaN in any component fails);
-//   DMP (lohi != null): every subcell inside [lo_v, hi_v], tested exactly on
-//        the per-variable extremes (min >= lo and max <= hi).
-// Writes the per-variable min / max to mm[2v], mm[2v+1] and, when lam != null,
-// the largest wave speed max_k |v_k| + c (FP32 speeds with f32speed).  Returns
-// (block-uniform) whether any check failed.  `red` needs (blockDim/32 + 1) * (2 nvar + 1) doubles.
-template <int D>
-__device__ __forceinline__ bool check_subcells(const double* __restrict__ vs, int nsub,
-                                               const double* lohi, double gamma, double* mm,
-                                               double* lam, double* red, bool f32speed = false,
-                                               float g2f = 0.0f) {
+//   per-variable extremes and, with `speed`, the largest wave speed
+//        max_k |v_k| + c (FP32 speeds with f32speed) as keys in
+//        r[2 v] = ~min, r[2 v + 1] = max, r[2 nvar].
+// Returns whether PAD failed on a subcell of this thread.
+template <int D, typename Value>
+__device__ __forceinline__ bool scan_subcells(Value value, int nsub, double gamma, bool speed,
+                                              bool f32speed, float g2f, int tid, int nth,
+                                              long long* r) {
   constexpr int NV = D + 2, K = 2 * NV + 1;
   bool bad = false;
-  long long r[K];
 #pragma unroll
   for (int j = 0; j < K; ++j) r[j] = LLONG_MIN;
-  for (int s = threadIdx.x; s < nsub; s += blockDim.x) {
+  for (int s = tid; s < nsub; s += nth) {
     double Q[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-      Q[v] = vs[v * nsub + s];
+      Q[v] = value(v, s);
       const long long k = ord_key(Q[v]);
       r[2 * v] = max(r[2 * v], ~k);          // ~k reverses the order: max of ~k = ~min k
       r[2 * v + 1] = max(r[2 * v + 1], k);
@@ -1367,49 +1442,66 @@ __device__ __forceinline__ bool check_subcells(const double* __restrict__ vs, in
     const double pe = Q[D + 1] * Q[0] - 0.5 * kin;
     // the two PAD comparisons as exact integer tests
     bad = bad || !(positive_f64(Q[0]) && positive_f64(pe));
-    if (lam)
+    if (speed)
       r[2 * NV] = max(r[2 * NV], speed_key(f32speed ? wave_speed_f<D>(Q, pe, g2f) : wave_speed<D>(Q, gamma)));
   }
+  return bad;
+}
+
+// Block version: the scan, the DMP test (lohi != null: the keys of the interval
+// [lo_v, hi_v], tested exactly on the per-variable extremes) and the results:
+// min / max to mm[2v], mm[2v+1], the largest speed to *lam (lam != null).
+// Returns (block-uniform) whether any check failed.  `red` needs
+// (blockDim/32 + 1) * (2 nvar + 1) doubles.
+template <int D, typename Value>
+__device__ __forceinline__ bool check_values(Value value, int nsub, const long long* lohi, double gamma,
+                                             double* mm, double* lam, double* red, bool f32speed,
+                                             float g2f) {
+  constexpr int NV = D + 2, K = 2 * NV + 1;
+  long long r[K];
+  bool bad = scan_subcells<D>(value, nsub, gamma, lam != nullptr, f32speed, g2f, threadIdx.x, blockDim.x, r);
   bad = __syncthreads_or(bad);
   const long long* res = block_max_keys<K>(r, reinterpret_cast<long long*>(red));
-  double mn[NV], mx[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    mn[v] = ord_val(~res[2 * v]);
-    mx[v] = ord_val(res[2 * v + 1]);
-  }
   if (lohi) {
-    // the DMP test on the extremes, by one warp (the others would repeat it)
-    int dmp = 0;
-    if (threadIdx.x < 32) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v)
-        dmp |= !((mn[v] >= lohi[2 * v]) && (mx[v] <= lohi[2 * v + 1]));
-    }
-    bad = __syncthreads_or(bad || dmp);
+    for (int v = 0; v < NV; ++v) bad = bad || !(~res[2 * v] >= lohi[2 * v] && res[2 * v + 1] <= lohi[2 * v + 1]);
   }
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      mm[2 * v] = mn[v];
-      mm[2 * v + 1] = mx[v];
-    }
-    if (lam) *lam = ord_val(res[2 * NV]);
-  }
+  if (threadIdx.x < 2 * NV) mm[threadIdx.x] = ord_val(threadIdx.x & 1 ? res[threadIdx.x] : ~res[threadIdx.x]);
+  if (threadIdx.x == 0 && lam) *lam = ord_val(res[2 * NV]);
   return bad;
+}
+
+template <int D>
+__device__ __forceinline__ bool check_subcells(const double* __restrict__ vs, int nsub,
+                                               const long long* lohi, double gamma, double* mm,
+                                               double* lam, double* red, bool f32speed = false,
+                                               float g2f = 0.0f) {
+  return check_values<D>([vs, nsub](int v, int s) { return vs[v * nsub + s]; }, nsub, lohi, gamma, mm,
+                         lam, red, f32speed, g2f);
 }
 
 // ---------------------------------------------------------------------------
 // K3 + K4 corrector and detector: one cell per block.
 // ---------------------------------------------------------------------------
+// Stages of the projection per variable: u (n^D), after the x pass (Ns
+// n^(D-1)), after the y pass, after the z pass.  The two buffers hold the even
+// and the odd ones, in FP64 or (the step's change) in FP32.
+template <int D, int N>
+struct ProjStages {
+  using DM = Dims<D, N>;
+  static constexpr int S0 = DM::ND, S1 = DM::Ns * ipow(DM::n, D - 1);
+  static constexpr int S2 = (D >= 2) ? DM::Ns * DM::Ns * ipow(DM::n, D - 2) : 0;
+  static constexpr int S3 = (D == 3) ? DM::NSD : 0;
+  static constexpr int SA = S0 > S2 ? S0 : S2, SB = S1 > S3 ? S1 : S3;
+};
+
 template <int D, int N>
 __host__ __device__ constexpr size_t correct_smem_bytes() {
   using DM = Dims<D, N>;
-  const int big = DM::NSD > DM::ND * 4 ? DM::NSD : DM::ND * 4;
-  // + the face terms' weights (2 d n doubles) and the FP32 copy of P1 (Ns n
-  // floats) for the projection of the step's change
-  return (size_t)(2 * DM::NV * (DM::NSD > big ? DM::NSD : big) + DM::Ns * DM::n + 4 * DM::NV + 128 +
-                  2 * D * DM::n + (DM::Ns * DM::n + 1) / 2) *
+  // the two stages, P1 (fixed point), the DMP interval, extremes, reductions
+  // and the face terms' weights (2 d n doubles)
+  return (size_t)(DM::NV * (ProjStages<D, N>::SA + ProjStages<D, N>::SB) + DM::Ns * DM::n + 4 * DM::NV +
+                  128 + 2 * D * DM::n) *
          sizeof(double);
 }
 
@@ -1418,23 +1510,19 @@ __host__ __device__ constexpr size_t correct_smem_bytes() {
 template <int D, int N>
 __global__ void __launch_bounds__(128, 8) k_correct_detect(Batch bt) {
   using DM = Dims<D, N>;
+  using ST = ProjStages<D, N>;
   constexpr int n = DM::n, NV = DM::NV, ND = DM::ND, NF = DM::NF, Ns = DM::Ns, NSD = DM::NSD;
-  constexpr int BUF = (DM::NSD > DM::ND * 4 ? DM::NSD : DM::ND * 4);
   extern __shared__ double sm[];
-  double* A = sm;                     // NV * BUF
-  double* B = A + NV * BUF;           // NV * BUF
-  FxOp* P1x = reinterpret_cast<FxOp*>(B + NV * BUF);   // Ns * n
-  double* lohi = reinterpret_cast<double*>(P1x + Ns * n);   // 2 NV
-  double* mm = lohi + 2 * NV;         // 2 NV
+  double* A = sm;                     // NV * SA
+  double* B = A + NV * ST::SA;        // NV * SB
+  FxOp* P1x = reinterpret_cast<FxOp*>(B + NV * ST::SB);            // Ns * n
+  long long* lohi = reinterpret_cast<long long*>(P1x + Ns * n);    // 2 NV
+  double* mm = reinterpret_cast<double*>(lohi + 2 * NV);           // 2 NV
   double* red = mm + 2 * NV;          // 128
   double* cw = red + 128;             // 2 D n: [k][side][a] dt/dx_k phi_side(a) / w_a
-  float* P1f = reinterpret_cast<float*>(cw + 2 * D * n);   // Ns * n
   const int tid = threadIdx.x, nth = blockDim.x;
   const Ops* o = bt.pps[0]->ops;
-  for (int i = tid; i < Ns * n; i += nth) {
-    P1x[i] = o->P1x[i];
-    P1f[i] = (float)o->P1[i];
-  }
+  for (int i = tid; i < Ns * n; i += nth) P1x[i] = o->P1x[i];
   const FxMat P1m = {P1x, o->gP1, o->P1};
   __syncthreads();
   for (long long g = blockIdx.x; g < bt.pre[bt.n]; g += gridDim.x) {
@@ -1469,8 +1557,8 @@ __global__ void __launch_bounds__(128, 8) k_correct_detect(Batch bt) {
     double* vkeep = p.b.vstar ? p.b.vstar + cell * (size_t)(NV * NSD) : nullptr;
     const bool delta = vkeep && p.b.vok[cell] && (p.stamp & 15) != 0;
     const double* Un = p.b.U[p.cur] + cell * (NV * ND);
-    float* dA = reinterpret_cast<float*>(B);          // FP32 change, then its projection
-    float* dB = dA + NV * BUF;
+    float* dA = reinterpret_cast<float*>(A);          // FP32 change, then its projection
+    float* dB = reinterpret_cast<float*>(B);
     // the face terms' weights of this cell's step, one product each (the
     // previous cell's readers passed several barriers since)
     for (int q = tid; q < 2 * D * n; q += nth) {
@@ -1495,30 +1583,36 @@ __global__ void __launch_bounds__(128, 8) k_correct_detect(Batch bt) {
         acc = fma(-cw[(2 * k + 1) * n + ak], Ghi, acc);
         acc = fma(cw[2 * k * n + ak], Glo, acc);
       }
-      A[e] = acc;
       Uo[e] = acc;
       if (delta) dA[e] = narrow_f64_rz(acc - Un[e]);    // (integer pipe; toward zero)
-    }
-    __syncthreads();
-    double* vs;
-    if (delta) {
-      const float* dv = apply_ct<D, NV, n, Ns, float>(dA, dB, P1f, tid, nth);
-      for (int e = tid; e < NV * NSD; e += nth) {
-        const double x = vkeep[e] + widen_f32(dv[e]);
-        A[e] = x;
-        vkeep[e] = x;
-      }
-      vs = A;
-    } else {
-      vs = apply_fx<D, NV, n, Ns>(A, B, P1m, tid, nth);
-      if (vkeep)
-        for (int e = tid; e < NV * NSD; e += nth) vkeep[e] = vs[e];
+      else A[e] = acc;
     }
     dmp_interval<D>(p, p.b.cmm[p.cur], ijk, lohi);
     __syncthreads();
     double lam = 0.0;
-    const bool bad = check_subcells<D>(vs, NSD, lohi, p.gamma, mm, p.lam_mode ? &lam : nullptr, red,
-                                       p.prec == ADG_PREC_MIXED_FP32, p.gam2f);
+    bool bad;
+    if (delta) {
+      // the projected change is added to the kept averages as the scan reads them
+      const float* dv = project_f<D, N, false>(dA, dB, tid, nth);
+      auto value = [vkeep, dv](int v, int s) {
+        const int e = v * NSD + s;
+        const double x = vkeep[e] + widen_f32(dv[e]);
+        vkeep[e] = x;
+        return x;
+      };
+      bad = check_values<D>(value, NSD, lohi, p.gamma, mm, p.lam_mode ? &lam : nullptr, red,
+                            p.prec == ADG_PREC_MIXED_FP32, p.gam2f);
+    } else {
+      const double* vs = apply_fx<D, NV, n, Ns>(A, B, P1m, tid, nth);
+      auto value = [vkeep, vs](int v, int s) {
+        const int e = v * NSD + s;
+        const double x = vs[e];
+        if (vkeep) vkeep[e] = x;
+        return x;
+      };
+      bad = check_values<D>(value, NSD, lohi, p.gamma, mm, p.lam_mode ? &lam : nullptr, red,
+                            p.prec == ADG_PREC_MIXED_FP32, p.gam2f);
+    }
     if (tid == 0) {
       int slot = -1;
       if (bad || p.force) {
@@ -1554,62 +1648,23 @@ namespace adg {
 // ---------------------------------------------------------------------------
 constexpr int CD_WARPS = 4;
 
-template <int D, int NV, int NI, int NO, typename T>
-__device__ __forceinline__ T* apply_ct_warp(T* a, T* b, const T* M, int lane) {
-  apply_pass_ct<D, NV, NI, NO, 0, T>(a, b, M, lane, 32);
-  __syncwarp();
-  if (D == 1) return b;
-  apply_pass_ct<D, NV, NI, NO, 1, T>(b, a, M, lane, 32);
-  __syncwarp();
-  if (D == 2) return a;
-  apply_pass_ct<D, NV, NI, NO, 2, T>(a, b, M, lane, 32);
-  __syncwarp();
-  return b;
-}
-
-// Warp version of check_subcells: per-variable extremes, PAD, the DMP test on
-// the extremes against lohi (if given) and the largest wave speed; every lane
-// returns the results (mm[2v], mm[2v+1], *lam) and whether a check failed.
-template <int D>
-__device__ __forceinline__ bool check_subcells_warp(const double* __restrict__ vs, int nsub,
-                                                    const double* lohi, double gamma, double* mm,
-                                                    double* lam, bool f32speed, int lane,
-                                                    float g2f) {
+// Warp version of check_values; every lane returns the extremes mm, *lam and
+// whether a check failed.
+template <int D, typename Value>
+__device__ __forceinline__ bool check_values_warp(Value value, int nsub, const long long* lohi,
+                                                  double gamma, double* mm, double* lam, bool f32speed,
+                                                  int lane, float g2f) {
   constexpr int NV = D + 2, K = 2 * NV + 1;
-  bool bad = false;
   long long r[K];
+  bool bad = scan_subcells<D>(value, nsub, gamma, lam != nullptr, f32speed, g2f, lane, 32, r);
 #pragma unroll
-  for (int j = 0; j < K; ++j) r[j] = LLONG_MIN;
-  for (int s = lane; s < nsub; s += 32) {
-    double Q[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      Q[v] = vs[v * nsub + s];
-      const long long k = ord_key(Q[v]);
-      r[2 * v] = max(r[2 * v], ~k);
-      r[2 * v + 1] = max(r[2 * v + 1], k);
-    }
-    double kin = 0.0;
-#pragma unroll
-    for (int k = 0; k < D; ++k) kin += Q[1 + k] * Q[1 + k];
-    const double pe = Q[D + 1] * Q[0] - 0.5 * kin;
-    bad = bad || !(positive_f64(Q[0]) && positive_f64(pe));
-    if (lam)
-      r[2 * NV] = max(r[2 * NV], speed_key(f32speed ? wave_speed_f<D>(Q, pe, g2f) : wave_speed<D>(Q, gamma)));
-  }
-#pragma unroll
-  for (int j = 0; j < K; ++j)
-    for (int o = 16; o > 0; o >>= 1) r[j] = max(r[j], __shfl_xor_sync(0xffffffffu, r[j], o));
+  for (int j = 0; j < K; ++j) r[j] = warp_max_key(r[j]);
   bad = __any_sync(0xffffffffu, bad);
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
+    bad = bad || !(~r[2 * v] >= lohi[2 * v] && r[2 * v + 1] <= lohi[2 * v + 1]);
     mm[2 * v] = ord_val(~r[2 * v]);
     mm[2 * v + 1] = ord_val(r[2 * v + 1]);
-  }
-  if (lohi) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v)
-      bad = bad || !((mm[2 * v] >= lohi[2 * v]) && (mm[2 * v + 1] <= lohi[2 * v + 1]));
   }
   if (lam) *lam = ord_val(r[2 * NV]);
   return bad;
@@ -1618,23 +1673,14 @@ __device__ __forceinline__ bool check_subcells_warp(const double* __restrict__ v
 template <int D, int N>
 struct CdLayout {
   using DM = Dims<D, N>;
-  // sizes per variable of the projection's stages: u (n^D), after the x pass
-  // (Ns n^(D-1)), after the y pass (Ns^2 n^(D-2)), after the z pass (Ns^3)
-  static constexpr int S0 = DM::ND, S1 = DM::Ns * ipow(DM::n, D - 1);
-  static constexpr int S2 = (D >= 2) ? DM::Ns * DM::Ns * ipow(DM::n, D - 2) : 0;
-  static constexpr int S3 = (D == 3) ? DM::NSD : 0;
-  static constexpr int SA = S0 > S2 ? S0 : S2, SB = S1 > S3 ? S1 : S3;
-  // per warp: A [NV][SA] doubles (u*, then P(u*)), B (the FP64 projection's
-  // other stage, [NV][SB] doubles, or the FP32 projection of the change:
-  // [NV][SA] + [NV][SB] floats), face weights [2 D][n] doubles, lohi [2 NV]
-  static constexpr int A_DBL = DM::NV * SA;
-  static constexpr int B_DBL = (DM::NV * SB > (DM::NV * (SA + SB) + 1) / 2) ? DM::NV * SB
-                                                                            : (DM::NV * (SA + SB) + 1) / 2;
-  static constexpr int DB_FLT = DM::NV * SA;          // offset of the second FP32 stage
+  using ST = ProjStages<D, N>;
+  // per warp: the two stages of the projection, face weights [2 D][n], the keys
+  // of the DMP interval [2 NV]
+  static constexpr int A_DBL = DM::NV * ST::SA, B_DBL = DM::NV * ST::SB;
   static constexpr int CW_DBL = 2 * D * DM::n;
   static constexpr int WARP_DBL = A_DBL + B_DBL + CW_DBL + 2 * DM::NV;
-  // per block: P1 [Ns n] doubles and its FP32 copy
-  static constexpr int OPS_DBL = DM::Ns * DM::n + (DM::Ns * DM::n + 1) / 2;
+  // per block: P1 (fixed point)
+  static constexpr int OPS_DBL = DM::Ns * DM::n;
 };
 
 template <int D, int N>
@@ -1649,17 +1695,13 @@ __global__ void __launch_bounds__(32 * CD_WARPS) k_correct_detect_w(Batch bt) {
   constexpr int n = DM::n, NV = DM::NV, ND = DM::ND, NF = DM::NF, Ns = DM::Ns, NSD = DM::NSD;
   extern __shared__ double sm[];
   FxOp* P1x = reinterpret_cast<FxOp*>(sm);
-  float* P1f = reinterpret_cast<float*>(P1x + Ns * n);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double* A = sm + LY::OPS_DBL + w * LY::WARP_DBL;
   double* B = A + LY::A_DBL;
   double* cw = B + LY::B_DBL;          // [k][side][a]: dt/dx_k phi_side(a) / w_a
-  double* lohi = cw + LY::CW_DBL;
+  long long* lohi = reinterpret_cast<long long*>(cw + LY::CW_DBL);
   const Ops* o = bt.pps[0]->ops;
-  for (int i = threadIdx.x; i < Ns * n; i += 32 * CD_WARPS) {
-    P1x[i] = o->P1x[i];
-    P1f[i] = (float)o->P1[i];
-  }
+  for (int i = threadIdx.x; i < Ns * n; i += 32 * CD_WARPS) P1x[i] = o->P1x[i];
   const FxMat P1m = {P1x, o->gP1, o->P1};
   __syncthreads();
   const long long total = bt.pre[bt.n];
@@ -1696,8 +1738,8 @@ __global__ void __launch_bounds__(32 * CD_WARPS) k_correct_detect_w(Batch bt) {
     double* vkeep = p.b.vstar ? p.b.vstar + cell * (size_t)(NV * NSD) : nullptr;
     const bool delta = vkeep && p.b.vok[cell] && (p.stamp & 15) != 0;
     const double* Un = p.b.U[p.cur] + cell * (NV * ND);
-    float* dA = reinterpret_cast<float*>(B);
-    float* dB = dA + LY::DB_FLT;
+    float* dA = reinterpret_cast<float*>(A);
+    float* dB = reinterpret_cast<float*>(B);
     // the face terms' weights of this cell's step, one product each
     for (int q = lane; q < 2 * D * n; q += 32) {
       const int k = q / (2 * n), r = q - k * 2 * n;
@@ -1721,30 +1763,36 @@ __global__ void __launch_bounds__(32 * CD_WARPS) k_correct_detect_w(Batch bt) {
         acc = fma(-cw[(2 * k + 1) * n + ak], Ghi, acc);
         acc = fma(cw[2 * k * n + ak], Glo, acc);
       }
-      A[e] = acc;
       Uo[e] = acc;
       if (delta) dA[e] = narrow_f64_rz(acc - Un[e]);
-    }
-    __syncwarp();
-    double* vs;
-    if (delta) {
-      const float* dv = apply_ct_warp<D, NV, n, Ns, float>(dA, dB, P1f, lane);
-      for (int e = lane; e < NV * NSD; e += 32) {
-        const double x = vkeep[e] + widen_f32(dv[e]);
-        A[e] = x;
-        vkeep[e] = x;
-      }
-      vs = A;
-    } else {
-      vs = apply_fx<D, NV, n, Ns, true>(A, B, P1m, lane, 32);
-      if (vkeep)
-        for (int e = lane; e < NV * NSD; e += 32) vkeep[e] = vs[e];
+      else A[e] = acc;
     }
     if (lane < NV) dmp_interval_lane<D>(p, p.b.cmm[p.cur], ijk, lohi, lane);
     __syncwarp();
     double lam = 0.0, mm[2 * NV];
-    const bool bad = check_subcells_warp<D>(vs, NSD, lohi, p.gamma, mm, p.lam_mode ? &lam : nullptr,
-                                            p.prec == ADG_PREC_MIXED_FP32, lane, p.gam2f);
+    bool bad;
+    if (delta) {
+      // the projected change is added to the kept averages as the scan reads them
+      const float* dv = project_f<D, N, true>(dA, dB, lane, 32);
+      auto value = [vkeep, dv](int v, int s) {
+        const int e = v * NSD + s;
+        const double x = vkeep[e] + widen_f32(dv[e]);
+        vkeep[e] = x;
+        return x;
+      };
+      bad = check_values_warp<D>(value, NSD, lohi, p.gamma, mm, p.lam_mode ? &lam : nullptr,
+                                 p.prec == ADG_PREC_MIXED_FP32, lane, p.gam2f);
+    } else {
+      const double* vs = apply_fx<D, NV, n, Ns, true>(A, B, P1m, lane, 32);
+      auto value = [vkeep, vs](int v, int s) {
+        const int e = v * NSD + s;
+        const double x = vs[e];
+        if (vkeep) vkeep[e] = x;
+        return x;
+      };
+      bad = check_values_warp<D>(value, NSD, lohi, p.gamma, mm, p.lam_mode ? &lam : nullptr,
+                                 p.prec == ADG_PREC_MIXED_FP32, lane, p.gam2f);
+    }
     if (lane == 0) {
       int slot = -1;
       if (bad || p.force) {

@@ -1761,13 +1761,11 @@ __global__ void __launch_bounds__(128) k_lim_update(Batch bt, int pass) {
   extern __shared__ double sm[];
   double* A = sm;                 // NV * NSD
   double* B = A + NV * NSD;       // NV * NSD
-  FxOp* R1x = reinterpret_cast<FxOp*>(B + NV * NSD);        // n * Ns
-  double* mm = reinterpret_cast<double*>(R1x + n * Ns);     // 2 NV
+  double* R1 = B + NV * NSD;        // n * Ns
+  double* mm = R1 + n * Ns;         // 2 NV
   double* red = mm + 2 * NV;      // 128
   const int tid = threadIdx.x, nth = blockDim.x;
-  const Ops* o = bt.pps[0]->ops;
-  for (int i = tid; i < n * Ns; i += nth) R1x[i] = o->R1x[i];
-  const FxMat R1m = {R1x, o->gR1, o->R1};
+  for (int i = tid; i < n * Ns; i += nth) R1[i] = bt.pps[0]->ops->R1[i];
   for (long long tg = blockIdx.x; tg < bt.pre[bt.n]; tg += gridDim.x) {
     const LimItem it = lim_item(bt, tg);
     const Params& p = *bt.pps[it.s];
@@ -1850,7 +1848,7 @@ __global__ void __launch_bounds__(128) k_lim_update(Batch bt, int pass) {
     }
     // reconstruction R of the new subcell data
     __syncthreads();
-    double* u = apply_fx<D, NV, Ns, n>(A, B, R1m, tid, nth);
+    double* u = reconstruct<D, N>(A, B, R1, tid, nth);
     double* Uo = p.b.U[nxt] + cell * (NV * ND);
     for (int e = tid; e < NV * ND; e += nth) Uo[e] = u[e];
     if (tid == 0 && p.b.vok) p.b.vok[cell] = 0;     // P(R(v)) is not v: recompute next step
@@ -1991,17 +1989,15 @@ __global__ void __launch_bounds__(128) k_lim_fallback(Batch bt) {
   double* A = blk + NV * NB;        // NV * NSD
   double* B = A + NV * NSD;         // NV * NSD
   double* F = B + NV * NSD;         // NV * NFK  sub-face fluxes of one axis
-  FxOp* R1x = reinterpret_cast<FxOp*>(F + NV * NFK);        // n * Ns
-  double* P1 = reinterpret_cast<double*>(R1x + n * Ns);     // Ns * n
+  double* R1 = F + NV * NFK;        // n * Ns
+  double* P1 = R1 + n * Ns;         // Ns * n
   double* mm = P1 + Ns * n;         // 2 NV
   double* red = mm + 2 * NV;        // 128
   const int tid = threadIdx.x, nth = blockDim.x;
-  const Ops* o = bt.pps[0]->ops;
   for (int i = tid; i < n * Ns; i += nth) {
-    R1x[i] = o->R1x[i];
-    P1[i] = o->P1[i];
+    R1[i] = bt.pps[0]->ops->R1[i];
+    P1[i] = bt.pps[0]->ops->P1[i];
   }
-  const FxMat R1m = {R1x, o->gR1, o->R1};
   for (long long fg = blockIdx.x; fg < bt.pre[bt.n]; fg += gridDim.x) {
     const int sidx = batch_state(bt, fg);
     const Params& p = *bt.pps[sidx];
@@ -2104,7 +2100,7 @@ __global__ void __launch_bounds__(128) k_lim_fallback(Batch bt) {
     }
     if (tid < 2 * NV) p.b.cmm[nxt][cell * 2 * NV + tid] = mm[tid];
     __syncthreads();
-    double* u = apply_fx<D, NV, Ns, n>(A, B, R1m, tid, nth);
+    double* u = reconstruct<D, N>(A, B, R1, tid, nth);
     double* Uo = p.b.U[nxt] + cell * (NV * ND);
     for (int e = tid; e < NV * ND; e += nth) Uo[e] = u[e];
     if (tid == 0 && p.b.vok) p.b.vok[cell] = 0;     // P(R(v)) is not v: recompute next step
@@ -2143,14 +2139,12 @@ __global__ void __launch_bounds__(128) k_lim_refix(Batch bt) {
   extern __shared__ double sm[];
   double* A = sm;                   // NV * NSD
   double* B = A + NV * NSD;         // NV * NSD
-  FxOp* R1x = reinterpret_cast<FxOp*>(B + NV * NSD);        // n * Ns
-  double* mm = reinterpret_cast<double*>(R1x + n * Ns);     // 2 NV
+  double* R1 = B + NV * NSD;        // n * Ns
+  double* mm = R1 + n * Ns;         // 2 NV
   double* red = mm + 2 * NV;        // 128
   __shared__ int fbslot[6];         // slot of the fallback neighbour per face, -1: none
   const int tid = threadIdx.x, nth = blockDim.x;
-  const Ops* o = bt.pps[0]->ops;
-  for (int i = tid; i < n * Ns; i += nth) R1x[i] = o->R1x[i];
-  const FxMat R1m = {R1x, o->gR1, o->R1};
+  for (int i = tid; i < n * Ns; i += nth) R1[i] = bt.pps[0]->ops->R1[i];
   for (long long fg = blockIdx.x; fg < bt.pre[bt.n]; fg += gridDim.x) {
     const int sidx = batch_state(bt, fg);
     const Params& p = *bt.pps[sidx];
@@ -2221,7 +2215,7 @@ __global__ void __launch_bounds__(128) k_lim_refix(Batch bt) {
     }
     if (tid < 2 * NV) p.b.cmm[nxt][cell * 2 * NV + tid] = mm[tid];
     __syncthreads();
-    double* u = apply_fx<D, NV, Ns, n>(A, B, R1m, tid, nth);
+    double* u = reconstruct<D, N>(A, B, R1, tid, nth);
     double* Uo = p.b.U[nxt] + cell * (NV * ND);
     for (int e = tid; e < NV * ND; e += nth) Uo[e] = u[e];
     if (tid == 0 && p.b.vok) p.b.vok[cell] = 0;     // P(R(v)) is not v: recompute next step

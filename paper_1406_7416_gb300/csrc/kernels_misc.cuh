@@ -18,16 +18,16 @@ __global__ void __launch_bounds__(128) k_load_detect(Params p, const double* __r
   double* A = sm;
   double* B = A + NV * NSD;
   FxOp* P1x = reinterpret_cast<FxOp*>(B + NV * NSD);
-  FxOp* R1x = P1x + Ns * n;
-  double* lohi = reinterpret_cast<double*>(R1x + n * Ns);
-  double* mm = lohi + 2 * NV;
+  double* R1 = reinterpret_cast<double*>(P1x + Ns * n);
+  long long* lohi = reinterpret_cast<long long*>(R1 + n * Ns);
+  double* mm = reinterpret_cast<double*>(lohi + 2 * NV);
   double* red = mm + 2 * NV;
   const int tid = threadIdx.x, nth = blockDim.x;
   for (int i = tid; i < Ns * n; i += nth) {
     P1x[i] = p.ops->P1x[i];
-    R1x[i] = p.ops->R1x[i];
+    R1[i] = p.ops->R1[i];
   }
-  const FxMat P1m = {P1x, p.ops->gP1, p.ops->P1}, R1m = {R1x, p.ops->gR1, p.ops->R1};
+  const FxMat P1m = {P1x, p.ops->gP1, p.ops->P1};
   __shared__ int s_slot;
   const int cur = p.cur;
   for (long long cell = blockIdx.x; cell < p.geo.cells; cell += gridDim.x) {
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(128) k_load_detect(Params p, const double* __r
     }
     __syncthreads();
     check_subcells<D>(A, NSD, nullptr, p.gamma, mm, &lam, red);
-    double* u = apply_fx<D, NV, Ns, n>(A, B, R1m, tid, nth);
+    double* u = reconstruct<D, N>(A, B, R1, tid, nth);
     for (int e = tid; e < NV * ND; e += nth) U[e] = u[e];
     if (tid == 0) {
       p.b.beta[cur][cell] = 1;

@@ -66,6 +66,11 @@ static inline cudaError_t upload_picard_constants_here(int N, const Ops& o) {
   if (e != cudaSuccess) return e;
   e = cudaMemcpyToSymbol(c_Ktf, o.Ktf, sizeof(float) * n * n, sizeof(float) * (size_t)N * MAXN * MAXN);
   if (e != cudaSuccess) return e;
+  float p1[MAXNS * MAXN];
+  const int np = (2 * N + 1) * n;
+  for (int i = 0; i < np; ++i) p1[i] = (float)o.P1[i];
+  e = cudaMemcpyToSymbol(c_P1f, p1, sizeof(float) * np, sizeof(float) * (size_t)N * MAXNS * MAXN);
+  if (e != cudaSuccess) return e;
   float d3[9], k3[9];
   for (int i = 0; i < 9; ++i) {
     d3[i] = (float)o.D3[i];

@@ -202,7 +202,6 @@ void build_ops(int N, Ops* o) {
       o->Mt[a * Ns + s] = (double)(P1[s * n + a] / (Ns * w[a]));
     }
   o->gP1 = fixed_point(o->P1, Ns, n, o->P1x);
-  o->gR1 = fixed_point(o->R1, n, Ns, o->R1x);
   // composite rule of the initial projection: Ns subintervals x (N+2) points
   {
     ld xq[MAXN + 1], wq[MAXN + 1];
