@@ -199,7 +199,10 @@ extern "C" {
                                                             3D): one warp per cell for
                                                             the FP32 sweeps, 1, 2 or 4
                                                             cells per block sharing
-                                                            the FP64 terms
+                                                            the FP64 terms (2 in 2D:
+                                                            one thread per spatial
+                                                            node, several cells per
+                                                            block)
                                        ADG_PRED_WARP4_TC    the same, with the sweeps'
                                                             contractions on the tensor
                                                             pipe (TF32 operands split

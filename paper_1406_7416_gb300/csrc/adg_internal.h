@@ -208,7 +208,8 @@ struct StepLaunch {
 //                   FP32 kernels whose default is their launch bound: 64);
 //   PRED_WARP1/2/4  mixed precision with the split final stage: one warp per
 //                   cell for the FP32 sweeps, 1, 2 or 4 cells per block sharing
-//                   the FP64 terms (k_predictor_split);
+//                   the FP64 terms (k_predictor_split); 2 in 2D: one
+//                   thread per spatial node (k_predictor_node);
 //   PRED_WARP4_TC   the same with the sweeps' contractions on the tensor pipe
 //                   (3 x TF32 mma.sync, FP32-accurate).
 enum PredShapeId { PRED_BLOCK = 0, PRED_BLOCK_ALT = 1, PRED_WARP2 = 2, PRED_WARP4 = 3,

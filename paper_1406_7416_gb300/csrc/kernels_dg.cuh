@@ -45,11 +45,12 @@ struct PredShape {
   static constexpr int threads = wide ? 256 : (narrow3 ? 160 : 128);   // launched per block
   static constexpr int bound = (MIXED && !wide) ? threads : 256;       // __launch_bounds__ maximum
   // registers: <= 102 for the narrow mixed kernels (five 128- or four
-  // 160-thread blocks per SM), <= 128 otherwise (two 256-thread or four
-  // 128-thread blocks), except the FP64 kernel at 2D N >= 6, which would spill
-  // under that cap
+  // 160-thread blocks per SM), <= 128 for the wide ones (two 256-thread or four
+  // 128-thread blocks); <= 64 in FP64 up to N = 5, where the phases' barriers
+  // want more blocks beside each other (256^2 N = 5: 6.72 ms per step at 96
+  // registers, 6.37 at 80, 5.97 at 64, 6.12 at 48); no cap above (no difference)
   static constexpr int min_blocks =
-      narrow3 ? 4 : ((MIXED && !wide) ? 5 : ((!MIXED && D == 2 && N >= 6) ? 1 : 2));
+      narrow3 ? 4 : ((MIXED && !wide) ? 5 : (MIXED ? 2 : ((D == 2 && N >= 6) ? 1 : 4)));
 };
 
 // ---------------------------------------------------------------------------

@@ -19,6 +19,8 @@
 // products per tile: FP32-accurate).
 #pragma once
 
+#include <type_traits>
+
 #include "kernels_dg.cuh"
 
 namespace adg {
@@ -539,6 +541,343 @@ __global__ void __launch_bounds__(32 * W) k_predictor_split(Batch bt) {
       p.b.U[1 - p.cur][s_cell[ww] * (NV * ND) + e] = acc;
     }
     __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The same predictor in 2D with one thread per spatial node (PRED_WARP2 in 2D):
+// a block takes W cells, W n^2 threads, and a sweep is two phases.  Derivatives
+// run by lines in place, F_x <- c_x D x_x F_x, F_y <- D x_y F_y, so the axes need
+// no order and no second array; then each thread forms S = F_x + c_y F_y at its
+// node's time nodes in registers, solves for them (Ktau) and writes the new
+// fluxes of each time node straight from q, which never exists in memory.  A
+// warp per cell went through shared memory for S and for q as well, with 144
+// lines or 216 nodes per phase on 32 lanes, and its 12 KB per cell (8 KB here)
+// held an SM to 18 warps.  The operations of every output and their order are
+// those of k_predictor_split: the same bits.
+//
+// Measured (GB300), predictor per step: 512^2 N = 5 3.49 -> 3.03 ms, 350 x 100
+// N = 5 0.485 -> 0.415, 128^2 N = 5 0.236 -> 0.200; 10.0k -> 7.5k instructions
+// per cell; at 256^2 five cells per block at 80 registers 774 us, at 64 786, four
+// cells 814, three 829.
+// ---------------------------------------------------------------------------
+template <int N>
+struct NodeLayout {
+  using DM = Dims<2, N>;
+  static constexpr int n = DM::n, ND = DM::ND, NST = DM::NST;
+  // cells per block: W n^2 nodes fill the block's warps (94% to 100%)
+  static constexpr int W = N == 5 ? 5 : (N == 4 ? 5 : (N == 3 ? 8 : (N == 2 ? 14 : 32)));
+  static constexpr int threads = (W * ND + 31) / 32 * 32;
+  static constexpr int blocks = 65536 / (threads * 80);     // at 80 registers
+  // per cell: u (FP64 [4][ND]), then the fluxes (FP32 [2][4][NST]); after the
+  // last sweep dq in F_x's place and fbar (FP64 [2][4][ND]) behind it
+  static constexpr int FLT = 8 * NST > 4 * NST + 16 * ND ? 8 * NST : 4 * NST + 16 * ND;
+  static constexpr size_t cell_bytes = (size_t)4 * ND * 8 + (size_t)FLT * 4;
+  static constexpr size_t bytes = (size_t)(n * n + 2 * n) * 8 + (size_t)((3 * n + 1) / 2 * 2) * 4 + W * cell_bytes;
+};
+
+template <int N>
+__global__ void __launch_bounds__(NodeLayout<N>::threads, NodeLayout<N>::blocks) k_predictor_node(Batch bt) {
+  using LY = NodeLayout<N>;
+  constexpr int n = LY::n, NV = 4, ND = LY::ND, NST = LY::NST, NF = n, NT = ND, W = LY::W, T = LY::threads;
+  extern __shared__ double sm[];
+  double* Mv = sm;
+  double* ph0 = Mv + n * n;
+  double* ph1 = ph0 + n;
+  float* ph0f = reinterpret_cast<float*>(ph1 + n);
+  float* ph1f = ph0f + n;
+  float* wf = ph1f + n;
+  unsigned char* cells0 = reinterpret_cast<unsigned char*>(ph0f + (3 * n + 1) / 2 * 2);
+  __shared__ const Params* s_pp[W];
+  __shared__ long long s_cell[W];
+  __shared__ int s_it[W];                 // sweeps of the cell (0: no cell, or its state idles)
+  __shared__ float s_cx[W];
+  const int tid = threadIdx.x;
+  const Ops* o = bt.pps[0]->ops;      // every state of a batch has degree N
+  for (int i = tid; i < n * n; i += T) Mv[i] = o->Mvol[i];
+  for (int i = tid; i < n; i += T) {
+    ph0[i] = o->phi0[i];
+    ph1[i] = o->phi1[i];
+    ph0f[i] = (float)o->phi0[i];
+    ph1f[i] = (float)o->phi1[i];
+    wf[i] = (float)o->w[i];
+  }
+  // this thread's node
+  const int wn = tid / ND < W ? tid / ND : W - 1, node = tid - wn * ND;
+  const bool mine = tid < W * ND;
+  double* u = reinterpret_cast<double*>(cells0 + (size_t)wn * LY::cell_bytes);
+  float* F = reinterpret_cast<float*>(u + NV * ND);       // [k][v][NST]
+
+  // This thread's lines of n space-time nodes, the same along both axes in every
+  // sweep: line vr of the NV NT of cell w starts at n vr along x and at
+  // n vr - (n - 1)(vr % n) along y (offsets within a cell's variables).
+  constexpr int LC = NV * NT, NLINE = (W * LC + T - 1) / T;
+  int lw[NLINE], lv[NLINE];
+#pragma unroll
+  for (int i = 0; i < NLINE; ++i) {
+    const int e = tid + i * T;
+    lw[i] = e < W * LC ? e / LC : -1;
+    lv[i] = e % LC;
+  }
+  // one line of the derivative phase, in place
+  auto line = [](float* f, auto stride, float c, bool scale) {
+    constexpr int st = decltype(stride)::value;
+    float x[n];
+#pragma unroll
+    for (int j = 0; j < n; ++j) x[j] = f[j * st];
+#pragma unroll
+    for (int a = 0; a < n; ++a) {
+      float acc = 0.0f;
+#pragma unroll
+      for (int j = 0; j < n; ++j) acc += c_Dmf[N][a * n + j] * x[j];
+      f[a * st] = scale ? c * acc : acc;
+    }
+  };
+  using StX = std::integral_constant<int, 1>;
+  using StY = std::integral_constant<int, n>;
+  auto fluxes = [&](int w) {
+    return reinterpret_cast<float*>(cells0 + (size_t)w * LY::cell_bytes + NV * ND * 8);
+  };
+
+  const long long total = bt.pre[bt.n];
+  const long long ngroups = (total + W - 1) / W;
+  for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
+    __syncthreads();
+    if (tid < W) {
+      const long long g = grp * W + tid;
+      int it = 0;
+      if (g < total) {
+        const int sidx = batch_state(bt, g);
+        const Params* pp = bt.pps[sidx];
+        s_pp[tid] = pp;
+        s_cell[tid] = g - bt.pre[sidx];
+        s_cx[tid] = (float)pp->b.coef[0];
+        if (*pp->b.dt > 0.0) it = pp->iters;
+      }
+      s_it[tid] = it;
+      // the DOF block of the cell this place takes next, into L2
+      constexpr unsigned UBYTES = NV * ND * sizeof(double);
+      const long long gn = g + (long long)gridDim.x * W;
+      if (gn < total) {
+        const int sn = batch_state(bt, gn);
+        const Params* pn = bt.pps[sn];
+        bulk_prefetch_l2(pn->b.U[pn->cur] + (gn - bt.pre[sn]) * (NV * ND), UBYTES);
+      }
+    }
+    __syncthreads();
+    const int n32 = mine ? s_it[wn] : 0;
+    int sweeps = 0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) sweeps = max(sweeps, s_it[w]);
+    float uf[NV], cy = 0.0f, gm1f = 0.0f;
+    // first sweep, from u (x) 1: fluxes and derivatives at time node 0 only
+    if (n32 > 0) {
+      const Params& p = *s_pp[wn];
+      cy = (float)p.b.coef[1];
+      gm1f = (float)(p.gamma - 1.0);
+      const double* Uc = p.b.U[p.cur] + s_cell[wn] * (NV * ND) + node;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const double x = Uc[v * ND];
+        u[v * ND + node] = x;
+        uf[v] = (float)x;
+      }
+      float Fl[2][NV];
+      euler_fluxes<2, float>(uf, gm1f, Fl);
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) F[(k * NV + v) * NST + node] = Fl[k][v];
+    }
+    __syncthreads();
+    for (int e = tid; e < W * NV * n; e += T) {
+      const int w = e / (NV * n), r = e - w * (NV * n), v = r / n, l = r - v * n;
+      if (s_it[w] > 0) {
+        float* f = fluxes(w) + v * NST;
+        line(f + n * l, StX{}, s_cx[w], true);
+        line(f + NV * NST + l, StY{}, 0.0f, false);
+      }
+    }
+    __syncthreads();
+    if (n32 > 1) {
+      // q_m = u - kappa_m S and its fluxes
+      float S[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) S[v] = F[v * NST + node] + cy * F[(NV + v) * NST + node];
+#pragma unroll
+      for (int m = 0; m < n; ++m) {
+        float kap = 0.0f;
+#pragma unroll
+        for (int j = 0; j < n; ++j) kap += c_Ktf[N][m * n + j];
+        float Q[NV], Fl[2][NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Q[v] = uf[v] - kap * S[v];
+        euler_fluxes<2, float>(Q, gm1f, Fl);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int v = 0; v < NV; ++v) F[(k * NV + v) * NST + node + m * ND] = Fl[k][v];
+      }
+    }
+    for (int it = 1; it < sweeps; ++it) {
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < NLINE; ++i) {
+        if (lw[i] >= 0 && it < s_it[lw[i]]) {
+          float* f = fluxes(lw[i]) + n * lv[i];
+          line(f, StX{}, s_cx[lw[i]], true);
+          line(f + NV * NST - (n - 1) * (lv[i] % n), StY{}, 0.0f, false);
+        }
+      }
+      __syncthreads();
+      if (it < n32 - 1) {
+        float S[NV][n];
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int m = 0; m < n; ++m)
+            S[v][m] = F[v * NST + node + m * ND] + cy * F[(NV + v) * NST + node + m * ND];
+#pragma unroll
+        for (int m = 0; m < n; ++m) {
+          float Q[NV], Fl[2][NV];
+#pragma unroll
+          for (int v = 0; v < NV; ++v) {
+            float acc = 0.0f;
+#pragma unroll
+            for (int j = 0; j < n; ++j) acc += c_Ktf[N][m * n + j] * S[v][j];
+            Q[v] = uf[v] - acc;
+          }
+          euler_fluxes<2, float>(Q, gm1f, Fl);
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) F[(k * NV + v) * NST + node + m * ND] = Fl[k][v];
+        }
+      }
+    }
+    // the last sweep's dq = -Ktau S, the time-averaged flux changes (in the
+    // groups of k_predictor_split) and fbar = F(u) + the changes
+    {
+      float S[NV][n];
+      if (n32 > 0) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+          for (int m = 0; m < n; ++m) {
+            const int at = node + (n32 > 1 ? m * ND : 0);
+            S[v][m] = F[v * NST + at] + cy * F[(NV + v) * NST + at];
+          }
+      }
+      __syncthreads();
+      if (n32 > 0) {
+        constexpr int TS = SplitLayout<2, N>::TSPLIT, MG = n / TS;
+        float dF[2][NV];
+#pragma unroll
+        for (int g = 0; g < TS; ++g) {
+          float acc[2][NV];
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) acc[k][v] = 0.0f;
+#pragma unroll
+          for (int mm = 0; mm < MG; ++mm) {
+            const int m = g * MG + mm;
+            float dQ[NV], G[2][NV];
+            float kap = 0.0f;
+#pragma unroll
+            for (int j = 0; j < n; ++j) kap += c_Ktf[N][m * n + j];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+              float a = 0.0f;
+#pragma unroll
+              for (int j = 0; j < n; ++j) a += c_Ktf[N][m * n + j] * S[v][j];
+              dQ[v] = n32 > 1 ? -a : 0.0f - kap * S[v][0];
+              F[v * NST + node + m * ND] = dQ[v];
+            }
+            euler_flux_delta<2>(uf, dQ, gm1f, G);
+            const float wm = wf[m];
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+              for (int v = 0; v < NV; ++v) acc[k][v] = __fadd_rn(acc[k][v], __fmul_rn(wm, G[k][v]));
+          }
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) dF[k][v] = g == 0 ? acc[k][v] : __fadd_rn(dF[k][v], acc[k][v]);
+        }
+        double Q[NV], Fl[2][NV];
+        double* fb = reinterpret_cast<double*>(F + NV * NST);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Q[v] = u[v * ND + node];
+        euler_fluxes<2, double>(Q, s_pp[wn]->gamma - 1.0, Fl);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+          for (int v = 0; v < NV; ++v) fb[(k * NV + v) * ND + node] = Fl[k][v] + widen_f32(dF[k][v]);
+      }
+    }
+    __syncthreads();
+    // trace(dq) in FP32 (the split trace layout of k_predictor), both faces from
+    // each line, whose index is the trace's; then trace(u) in FP64
+#pragma unroll
+    for (int i = 0; i < NLINE; ++i) {
+      if (lw[i] < 0 || s_it[lw[i]] == 0) continue;
+      double* tr = s_pp[lw[i]]->b.trace + s_cell[lw[i]] * (size_t)(4 * NV * NT) + NV * NF;
+      const float* d = fluxes(lw[i]) + n * lv[i];
+      float* t = reinterpret_cast<float*>(tr) + lv[i];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float* x = k == 0 ? d : d - (n - 1) * (lv[i] % n);
+        float a0 = 0.0f, a1 = 0.0f;
+#pragma unroll
+        for (int a = 0; a < n; ++a) {
+          a0 += ph0f[a] * x[a * (k == 0 ? 1 : n)];
+          a1 += ph1f[a] * x[a * (k == 0 ? 1 : n)];
+        }
+        t[(2 * k) * (2 * NV * NT)] = a0;
+        t[(2 * k + 1) * (2 * NV * NT)] = a1;
+      }
+    }
+    for (int e = tid; e < W * 2 * NV * NF; e += T) {
+      const int w = e / (2 * NV * NF);
+      int r = e - w * (2 * NV * NF);
+      if (s_it[w] == 0) continue;
+      const int k = r / (NV * NF);
+      r -= k * (NV * NF);
+      const int v = r / NF, l = r - v * NF;
+      const int st = k == 0 ? 1 : n;
+      const double* uu = reinterpret_cast<const double*>(cells0 + (size_t)w * LY::cell_bytes) + v * ND +
+                         n * l - (n - 1) * (l % st);
+      double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+      for (int a = 0; a < n; ++a) {
+        a0 += ph0[a] * uu[a * st];
+        a1 += ph1[a] * uu[a * st];
+      }
+      double* tr = s_pp[w]->b.trace + s_cell[w] * (size_t)(4 * NV * NT) + (2 * k) * (NV * NT);
+      tr[r] = a0;
+      tr[NV * NT + r] = a1;
+    }
+    // the volume part of the candidate, u + sum_k c_k Mvol x_k fbar_k, at this node
+    if (n32 > 0) {
+      const Params& p = *s_pp[wn];
+      const double* fb = reinterpret_cast<const double*>(F + NV * NST);
+      const int ix = node % n, iy = node / n;
+      const double cX = p.b.coef[0], cY = p.b.coef[1];
+      double* Uo = p.b.U[1 - p.cur] + s_cell[wn] * (NV * ND) + node;
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        double acc = u[v * ND + node], tx = 0.0, ty = 0.0;
+#pragma unroll
+        for (int j = 0; j < n; ++j) tx += Mv[ix * n + j] * fb[v * ND + iy * n + j];
+        acc += cX * tx;
+#pragma unroll
+        for (int j = 0; j < n; ++j) ty += Mv[iy * n + j] * fb[(NV + v) * ND + j * n + ix];
+        acc += cY * ty;
+        Uo[v * ND] = acc;
+      }
+    }
   }
 }
 

@@ -130,6 +130,20 @@ struct Launch {
     return cudaErrorInvalidValue;
   }
 
+  // The thread-per-node predictor (2D), persistent.
+  static cudaError_t launch_node(const Batch& cells, long long total, cudaStream_t s) {
+    if constexpr (D == 2 && kSplit) {
+      using LY = NodeLayout<N>;
+      const cudaError_t e = set_smem(k_predictor_node<N>, LY::bytes);
+      if (e != cudaSuccess) return e;
+      static const int grid_full = persistent_grid(k_predictor_node<N>, LY::threads, LY::bytes, 1LL << 40);
+      const long long groups = (total + LY::W - 1) / LY::W;
+      k_predictor_node<N><<<(int)(groups < grid_full ? groups : grid_full), LY::threads, LY::bytes, s>>>(cells);
+      return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;
+  }
+
   // The predictor in the launch shape sl.pred (PRED_*); shapes that do not
   // apply to the launch fall back to the block-per-cell kernel.
   static cudaError_t launch_predictor(const StepLaunch& sl, cudaStream_t s) {
@@ -138,7 +152,11 @@ struct Launch {
     const Batch cells{sl.pps, sl.n, sl.pre_cells};
     if (sl.prec == ADG_PREC_MIXED_FP32) {
       if (kSplit && sl.pred == PRED_WARP1) return launch_split<1, false>(cells, sl.total_cells, s);
-      if (kSplit && sl.pred == PRED_WARP2) return launch_split<2, false>(cells, sl.total_cells, s);
+      if constexpr (D == 2 && kSplit) {
+        if (sl.pred == PRED_WARP2) return launch_node(cells, sl.total_cells, s);
+      } else {
+        if (kSplit && sl.pred == PRED_WARP2) return launch_split<2, false>(cells, sl.total_cells, s);
+      }
       if (kSplit && sl.pred == PRED_WARP4) return launch_split<4, false>(cells, sl.total_cells, s);
       if (kSplit && sl.pred == PRED_WARP4_TC) return launch_split<4, true>(cells, sl.total_cells, s);
       const size_t sm = predictor_smem_bytes<D, N, true>();
