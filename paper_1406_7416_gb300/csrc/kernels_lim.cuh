@@ -451,52 +451,73 @@ __device__ __forceinline__ void weno3f(const float* u, const Ops* __restrict__ o
 // nodes (the new nodal index is the slowest digit).
 // T: the sweeps' precision (double; float for the mixed-precision FP32
 // reconstruction); the patch (input of the x sweep) is always FP64.
+//
+// One thread takes sweep_run neighbouring targets along K: their stencils share
+// all but one value each, and index arithmetic was 100 of the 234 instructions
+// that one FP32 target took by itself.  Measured (GB300), x / y / z: 40^3 N = 3
+// mixed 566 / 972 / 1982 -> 366 / 716 / 1840 us, 33 x 29 x 30 N = 3 FP64 4.1 / 8.5
+// / 17.6 -> 3.6 / 7.5 / 16.0 ms.  In 2D FP64, bound by the FP64 pipe with a
+// hundredth of the targets per cell, one target per thread stays: 146 patches
+// at N = 5 take 22 + 37 us, in runs of three 25 + 53.
+template <int D, typename T>
+constexpr int sweep_run = (D == 3 || sizeof(T) == sizeof(float)) ? 3 : 1;
+
 template <int D, int N, int K, typename T>
 __global__ void __launch_bounds__(256) k_lim_sweep(Batch bt, int pass) {
   using DM = Dims<D, N>;
-  constexpr int NV = DM::NV, L = DM::L, NE = DM::NE;
+  constexpr int NV = DM::NV, L = DM::L, NE = DM::NE, R = sweep_run<D, T>, NR = (NE + R - 1) / R;
   constexpr int I0 = (0 < K) ? NE : L, I1 = (1 < K) ? NE : L, I2 = (D < 3) ? 1 : ((2 < K) ? NE : L);
   constexpr int O0 = (0 <= K) ? NE : L, O1 = (1 <= K) ? NE : L, O2 = (D < 3) ? 1 : ((2 <= K) ? NE : L);
   constexpr int NNIN = ipow(3, K);
   constexpr int INSZ = I0 * I1 * I2 * NNIN;
   constexpr int OUTSZ = O0 * O1 * O2 * NNIN;          // elements, each producing 3 values
-  constexpr int STRIDE = ((K == 0) ? 1 : (K == 1 ? I0 : I0 * I1)) * NNIN;
+  constexpr int RUNS = OUTSZ / NE * NR;               // runs of targets
+  constexpr int R0 = K == 0 ? NR : O0, R1 = K == 1 ? NR : O1;
+  constexpr int STRIDE = ((K == 0) ? 1 : (K == 1 ? I0 : I0 * I1)) * NNIN;       // input, along K
+  constexpr int OSTRIDE = ((K == 0) ? 1 : (K == 1 ? O0 : O0 * O1)) * NNIN * 3;  // output
   const Ops* ops = bt.pps[0]->ops;
   for (long long eg = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-       eg < bt.pre[bt.n] * (NV * OUTSZ); eg += (long long)gridDim.x * blockDim.x) {
-    const long long t = eg / (NV * OUTSZ);
+       eg < bt.pre[bt.n] * (NV * RUNS); eg += (long long)gridDim.x * blockDim.x) {
+    const long long t = eg / (NV * RUNS);
     const LimItem it = lim_item(bt, t);
     const Params& p = *bt.pps[it.s];
-    T* out = reinterpret_cast<T*>(p.b.sweep[K]);
-    const long long e = eg - t * (NV * OUTSZ) + (long long)it.j * (NV * OUTSZ);
-    const long long jv = e / OUTSZ;
-    int r = (int)(e - jv * OUTSZ);
+    int r = (int)(eg - t * (NV * RUNS));
+    const int v = r / RUNS;
+    r -= v * RUNS;
+    const long long jv = (long long)it.j * NV + v;
     const int node = r % NNIN;
     r /= NNIN;
-    const int x0 = r % O0;
-    r /= O0;
-    const int x1 = r % O1;
-    const int x2 = r / O1;
+    int x0 = r % R0;
+    r /= R0;
+    int x1 = r % R1;
+    int x2 = r / R1;
+    const int first = R * (K == 0 ? x0 : (K == 1 ? x1 : x2));
+    if (K == 0) x0 = first;
+    if (K == 1) x1 = first;
+    if (K == 2) x2 = first;
     // input element whose axis-K index equals the output's (stencil x_K .. x_K + 4)
-    const int off = x0 + I0 * (x1 + I1 * x2);
-    const size_t src_off = jv * INSZ + (size_t)off * NNIN + node;
-    T u[5];
+    const size_t src_off = jv * INSZ + (size_t)(x0 + I0 * (x1 + I1 * x2)) * NNIN + node;
+    T u[R + 4];
     if (K == 0) {
       const double* src = p.b.patch + src_off;
 #pragma unroll
-      for (int q = 0; q < 5; ++q) u[q] = (T)src[q * STRIDE];
+      for (int q = 0; q < R + 4; ++q) u[q] = (T)(first + q < NE + 4 ? src[q * STRIDE] : 0.0);
     } else {
       const T* src = reinterpret_cast<const T*>(p.b.sweep[K > 0 ? K - 1 : 0]) + src_off;
 #pragma unroll
-      for (int q = 0; q < 5; ++q) u[q] = src[q * STRIDE];
+      for (int q = 0; q < R + 4; ++q) u[q] = first + q < NE + 4 ? src[q * STRIDE] : T(0);
     }
-    T res[3];
-    if constexpr (sizeof(T) == sizeof(double)) weno3(u, ops, res);
-    else weno3f(u, ops, res);
-    const int ooff = x0 + O0 * (x1 + O1 * x2);
-    T* dst = out + jv * (size_t)OUTSZ * 3 + (size_t)ooff * NNIN * 3 + node;
+    T* dst = reinterpret_cast<T*>(p.b.sweep[K]) + jv * (size_t)OUTSZ * 3 +
+             (size_t)(x0 + O0 * (x1 + O1 * x2)) * NNIN * 3 + node;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) dst[a * NNIN] = res[a];
+    for (int i = 0; i < R; ++i) {
+      if (first + i >= NE) break;
+      T res[3];
+      if constexpr (sizeof(T) == sizeof(double)) weno3(u + i, ops, res);
+      else weno3f(u + i, ops, res);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) dst[i * OSTRIDE + a * NNIN] = res[a];
+    }
   }
 }
 
@@ -1342,8 +1363,13 @@ __global__ void __launch_bounds__(128, 5) k_lim_predict_s3(Batch bt) {
 // Sub-face fluxes normal to axis k from the face traces of k_lim_predict_s3
 // (3D, FP32 subcell scheme, Rusanov): one warp per sub-face, lane t < 27
 // evaluates the flux at point t of the face (its two traces are contiguous
-// across the lanes), then the GL-weighted sum over the 27 points runs in
-// point order, as k_lim_flux accumulates it.  The result is stored in FP64.
+// across the lanes).  A warp takes FLUX_TURN sub-faces and then forms their
+// GL-weighted sums, one lane per (sub-face, variable), each over its 27 points
+// in point order, as k_lim_flux accumulates it (after every sub-face the 27
+// terms would run on five lanes: 892 -> 700 us per axis at 40^3, N = 3).  The
+// result is stored in FP64.
+constexpr int FLUX_TURN = 6;
+
 template <int N, int k>
 __global__ void __launch_bounds__(256) k_lim_flux_t(Batch bt, int pass) {
   pass = lim_pass(bt, pass);
@@ -1351,7 +1377,7 @@ __global__ void __launch_bounds__(256) k_lim_flux_t(Batch bt, int pass) {
   constexpr int NV = 5, Ns = TR::Ns, NFK = TR::NFK, NP = TR::NP;
   constexpr int WPB = 8;
   __shared__ float wts[NP];
-  __shared__ float gsum[WPB][NV][NP + 1];
+  __shared__ float gsum[WPB][FLUX_TURN * NV][NP + 1];
   const Ops* o = bt.pps[0]->ops;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (threadIdx.x < NP) {
@@ -1370,8 +1396,12 @@ __global__ void __launch_bounds__(256) k_lim_flux_t(Batch bt, int pass) {
   __syncthreads();
   const int t = lane < NP ? lane : NP - 1;                 // idle lanes mirror point 26
   const long long total = bt.pre[bt.n] * NFK;
-  for (long long item = (long long)blockIdx.x * WPB + w; item < total;
-       item += (long long)gridDim.x * WPB) {
+  const long long turns = (total + FLUX_TURN - 1) / FLUX_TURN;
+  for (long long turn = (long long)blockIdx.x * WPB + w; turn < turns; turn += (long long)gridDim.x * WPB) {
+#pragma unroll 1
+  for (int rd = 0; rd < FLUX_TURN; ++rd) {
+    const long long item = turn * FLUX_TURN + rd;
+    if (item >= total) break;
     const long long tg = item / NFK;
     const LimItem it = lim_item(bt, tg);
     const Params& p = *bt.pps[it.s];
@@ -1419,14 +1449,18 @@ __global__ void __launch_bounds__(256) k_lim_flux_t(Batch bt, int pass) {
     rusanov_f<3>(QL, QR, k, p.b.coef_f[7], G);
     if (lane < NP) {
 #pragma unroll
-      for (int v = 0; v < NV; ++v) gsum[w][v][lane] = G[v];
+      for (int v = 0; v < NV; ++v) gsum[w][rd * NV + v][lane] = G[v];
     }
+  }
     __syncwarp();
-    if (lane < NV) {
+    const long long item = turn * FLUX_TURN + lane / NV;
+    if (lane < FLUX_TURN * NV && item < total) {
+      const long long tg = item / NFK;
+      const LimItem it = lim_item(bt, tg);
       float acc = 0.0f;
 #pragma unroll
       for (int q = 0; q < NP; ++q) acc += wts[q] * gsum[w][lane][q];
-      p.b.fsub[k][((size_t)j * NV + lane) * NFK + e] = (double)acc;
+      bt.pps[it.s]->b.fsub[k][((size_t)it.j * NV + lane % NV) * NFK + (int)(item - tg * NFK)] = (double)acc;
     }
     __syncwarp();
   }

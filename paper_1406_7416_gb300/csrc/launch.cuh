@@ -372,7 +372,7 @@ struct Launch {
     } else if (traces) {
       if constexpr (D == 3) {
         // one warp per sub-face, persistent
-        const long long want = (ch * (Ns + 1) * DM::NSF + 7) / 8;
+        const long long want = (ch * (Ns + 1) * DM::NSF / FLUX_TURN + 8) / 8;
         static const int g0 = persistent_grid(k_lim_flux_t<N, 0>, 256, 0, 1LL << 40);
         static const int g1 = persistent_grid(k_lim_flux_t<N, 1>, 256, 0, 1LL << 40);
         static const int g2 = persistent_grid(k_lim_flux_t<N, 2>, 256, 0, 1LL << 40);
