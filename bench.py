@@ -103,19 +103,24 @@ def predictor_flops(D, N, iters, fp64_sweeps):
     """(fp64, fp32) flops of the predictor kernel for one cell: `iters` Picard
     sweeps, `fp64_sweeps` of them in FP64 and the others in FP32, then the
     final stage.  After an FP64 sweep (and in the FP64 path) the final stage
-    is FP64: fluxes at the space-time nodes, their time average, the volume
-    term and the face traces.  With no FP64 sweep it splits: F(u) at the
-    spatial nodes, the volume term and trace(u) in FP64; the flux changes at
-    the space-time nodes, their weighted time sum and trace(q - u) in FP32;
-    and the first sweep, from the time-constant u (x) 1, runs on the spatial
-    nodes only."""
+    is FP64.  Of the FP64 sweeps and their final stage the fluxes and the sums
+    are FP64 flops; the contractions (derivatives, time solve, time average,
+    volume term, traces) are fixed-point products on the integer pipes and not
+    counted.  With no FP64 sweep it splits: F(u) at the spatial nodes, the
+    volume term and trace(u) in FP64; the flux changes at the space-time nodes,
+    their weighted time sum and trace(q - u) in FP32.  The first sweep, from the
+    time-constant u (x) 1, runs on the spatial nodes only where it is FP64 or
+    split."""
     n, nv = N + 1, D + 2
     nst, nd, nf = n ** (D + 1), n ** D, n ** (D - 1)
     it = nst * flux_flops(D) + nv * nst * D * (2 * n + 2) + nv * nd * n * (2 * n + 1)
     vol = nv * nd * D * (2 * n + 2)
     if fp64_sweeps > 0:
-        final = nst * flux_flops(D) + D * nv * nd * 2 * n + vol + 2 * D * nv * nf * n * 2 * n
-        return fp64_sweeps * it + final, (iters - fp64_sweeps) * it
+        sweep64 = nst * flux_flops(D) + nv * nst * D
+        final = nst * flux_flops(D) + nv * nd * D
+        first64 = nd * flux_flops(D) + nv * nd * (D - 1) + nv * nst
+        f64 = (first64 + (iters - 1) * sweep64 if fp64_sweeps >= iters else fp64_sweeps * sweep64)
+        return f64 + final, max(0, iters - fp64_sweeps) * it
     final64 = nd * flux_flops(D) + D * nv * nd + vol + 2 * D * nv * nf * 2 * n
     final32 = (nst * flux_delta_flops(D) + D * nv * nst * 2 + 2 * D * nv * nf * n * 2 * n
                + nv * nst * n * 2)
