@@ -935,6 +935,12 @@ struct SubTraces2 {
 // picard_deriv_sub / picard_time_sub.  TRACES: the subcell's traces on the
 // sub-faces of the flux kernels (SubTraces2), each evaluated as k_lim_flux
 // evaluates it from the nodal values, instead of the nodal values.
+// Bound by instruction issue and the shuffles.  The traces go through shared
+// memory, one lane to a line and both its ends: by shuffles, with a third of
+// the lanes storing single floats under branches, they were 40% of the
+// instructions.  463 cells at N = 5: 68.1 -> 44.0 us (128 registers, two
+// blocks per SM; 80 registers 46.7, 64 registers 50.1); 512^2 limiter 1.36 ->
+// 1.10 ms per step.
 template <int N, bool TRACES>
 __global__ void __launch_bounds__(256) k_lim_predict_s2(Batch bt) {
   using DM = Dims<2, N>;
@@ -961,6 +967,9 @@ __global__ void __launch_bounds__(256) k_lim_predict_s2(Batch bt) {
       ph1[j] = (float)o->phi13[j];
     }
   }
+  constexpr int QS = NV * NST3 + 29;                    // the three subcells' nodes in different banks
+  __shared__ float nodal[TRACES ? 8 : 1][TRACES ? 3 * QS : 1];
+  __shared__ __align__(16) float* ends[TRACES ? 8 : 1][12];   // [subcell][axis][high, low end]
   const int wpb = blockDim.x >> 5;
   const long long total = bt.pre[bt.n] * NCROSS;
   const long long groups = (total + 2) / 3;
@@ -1042,37 +1051,43 @@ __global__ void __launch_bounds__(256) k_lim_predict_s2(Batch bt) {
           for (int m = 0; m < 3; ++m) dst[v * NST3 + m * ND3 + node] = q[m][v];
       }
     } else {
+      // the nodal values through shared memory; then a lane takes a whole line
+      // (its subcell gs, axis k and row w = point + 9 v, v its variable) and
+      // both its ends
       using TR = SubTraces2<N>;
-      float* trc = reinterpret_cast<float*>(p.b.qsub) + (size_t)j0 * TR::per_cell;
-      const int cc[2] = {sc % (Ns + 2), sc / (Ns + 2)};
+      float* sq = nodal[threadIdx.x >> 5];
+      float** dst = ends[threadIdx.x >> 5];
+      if (lane < 27) {
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int o = 1 - k;                              // the tangential axis
-        // (lanes of different subcells disagree here: every lane takes part in
-        // the shuffles and only writes when its subcell has these faces)
-        const bool faces = cc[o] >= 1 && cc[o] <= Ns;
-        const int ak = k == 0 ? a : b;
-        const int base = k == 0 ? sx : sy;
-        const int stk = k == 0 ? 1 : 3;
-        const int d = k == 0 ? b : a;                     // tangential digit
-        const int ft = (faces ? cc[o] - 1 : 0) * (k == 0 ? Ns + 1 : 1);
-        const int kmul = k == 0 ? 1 : Ns;
-        const bool wr_hi = live && faces && ak == 2 && cc[k] <= Ns;
-        const bool wr_lo = live && faces && ak == 0 && cc[k] >= 1;
-        // (offsets clamped into the cell's block when the lane does not write)
-        float* hi = trc + TR::offset(k, ft + (cc[k] <= Ns ? cc[k] : Ns) * kmul, 0);
-        float* lo = trc + TR::offset(k, ft + (cc[k] >= 1 ? cc[k] - 1 : 0) * kmul, 1);
+        for (int v = 0; v < NV; ++v)
 #pragma unroll
-        for (int m = 0; m < 3; ++m)
-#pragma unroll 2
-          for (int v = 0; v < NV; ++v) {
-            const float x0 = __shfl_sync(0xffffffffu, q[m][v], base);
-            const float x1 = __shfl_sync(0xffffffffu, q[m][v], base + stk);
-            const float x2 = __shfl_sync(0xffffffffu, q[m][v], base + 2 * stk);
-            if (wr_hi) hi[v * 9 + d + 3 * m] = ph1[0] * x0 + ph1[1] * x1 + ph1[2] * x2;
-            if (wr_lo) lo[v * 9 + d + 3 * m] = ph0[0] * x0 + ph0[1] * x1 + ph0[2] * x2;
-          }
+          for (int m = 0; m < 3; ++m) sq[g * QS + v * NST3 + m * ND3 + node] = q[m][v];
+        if (node < 2) {
+          const int ck = node == 0 ? sc % (Ns + 2) : sc / (Ns + 2);
+          const int co = node == 0 ? sc / (Ns + 2) : sc % (Ns + 2);
+          const bool faces = live && co >= 1 && co <= Ns;
+          const int ft = (co - 1) * (node == 0 ? Ns + 1 : 1), kmul = node == 0 ? 1 : Ns;
+          float* trc = reinterpret_cast<float*>(p.b.qsub) + (size_t)j0 * TR::per_cell;
+          dst[2 * (2 * g + node)] = faces && ck <= Ns ? trc + TR::offset(node, ft + ck * kmul, 0) : nullptr;
+          dst[2 * (2 * g + node) + 1] = faces && ck >= 1 ? trc + TR::offset(node, ft + (ck - 1) * kmul, 1) : nullptr;
+        }
       }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 7; ++i) {
+        const int li = i * 32 + lane;
+        if (li < 216) {
+          const int gk = li / 36, w = li - 36 * gk, r3 = w / 3, k = gk & 1;
+          const float* x = sq + (gk >> 1) * QS + (k == 0 ? 3 * w : 9 * r3 + (w - 3 * r3));
+          const int st = k == 0 ? 1 : 3;
+          float* hi = dst[2 * gk];
+          float* lo = dst[2 * gk + 1];
+          const float x0 = x[0], x1 = x[st], x2 = x[2 * st];
+          if (hi) hi[w] = ph1[0] * x0 + ph1[1] * x1 + ph1[2] * x2;
+          if (lo) lo[w] = ph0[0] * x0 + ph0[1] * x1 + ph0[2] * x2;
+        }
+      }
+      __syncwarp();
     }
   }
 }
