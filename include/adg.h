@@ -336,6 +336,9 @@ int adg_time(adg_state* st, double* t, int64_t* steps);
  *   (ADG_OPT_END_TIME); states past their end time idle.  CFL steps run as
  *   one CUDA graph, captured on the first and replayed while cfl is
  *   unchanged; each group's limiter passes loop on the device.
+ * Options set on a state (adg_set_option) count from the batch's next step;
+ * one that its launches depend on (ADG_OPT_FLUX, _FP64_SWEEPS, _PREDICTOR,
+ * _CASCADE, _SUBCELL_*) makes that step group the states again.
  * Asynchronous; errors of device-side conditions surface in adg_status of
  * the states. */
 typedef struct adg_batch adg_batch;

@@ -811,8 +811,25 @@ int ensure_lambda(adg_state* st) {
 
 }  // namespace
 
+// The options of a state that its launches' description holds.
+struct LaunchOptions {
+  int sub_fp64, sub_f32, sub_reg, flux, pred, split, cascade;
+  explicit LaunchOptions(const adg_state* st)
+      : sub_fp64(st->sub_fp64), sub_f32(st->sub_f32), sub_reg(st->sub_reg), flux(st->flux),
+        pred(effective_pred(st)), split(split_traces_of(st)), cascade(st->cascade) {}
+  // whether two states can share their launches
+  bool shared(const LaunchOptions& o) const {
+    return sub_fp64 == o.sub_fp64 && sub_f32 == o.sub_f32 && sub_reg == o.sub_reg && flux == o.flux &&
+           pred == o.pred;
+  }
+  bool operator==(const LaunchOptions& o) const {
+    return shared(o) && split == o.split && cascade == o.cascade;
+  }
+};
+
 struct adg_batch {
   std::vector<adg_state*> states;
+  std::vector<LaunchOptions> options;   // of each state, as grouped
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   struct Group {
@@ -840,11 +857,125 @@ void batch_free(adg_batch* b) {
   if (b->cap) cudaStreamDestroy(b->cap);
   if (b->body) cudaStreamDestroy(b->body);
   for (void* p : b->mem) cudaFree(p);
+  if (b->d_dts) cudaFree(b->d_dts);
   if (b->own_stream) {
     for (adg_state* st : b->states) st->stream = nullptr;
     cudaStreamDestroy(b->stream);
   }
   delete b;
+}
+
+// Groups of states that share their launches (equal dimension, degree,
+// precision and launch options), with the launch description of each; replaces
+// the former groups, whose step graph is dropped.
+int batch_group(adg_batch* b) {
+  if (b->stream) cudaStreamSynchronize(b->stream);
+  if (b->exec) cudaGraphExecDestroy(b->exec);
+  if (b->graph) cudaGraphDestroy(b->graph);
+  b->exec = nullptr;
+  b->graph = nullptr;
+  b->groups.clear();
+  for (void* p : b->mem) cudaFree(p);
+  b->mem.clear();
+  b->options.clear();
+  for (const adg_state* st : b->states) b->options.push_back(LaunchOptions(st));
+  const std::vector<adg_state*>& states = b->states;
+  const int count = (int)states.size();
+  std::vector<int> done(count, 0);
+  int off = 0;
+  for (int i = 0; i < count; ++i) {
+    if (done[i]) continue;
+    adg_batch::Group g;
+    g.rep = states[i];
+    for (int j = i; j < count; ++j) {
+      const adg_state* a = states[i];
+      const adg_state* c = states[j];
+      if (!done[j] && a->dim == c->dim && a->N == c->N && a->prec == c->prec &&
+          b->options[i].shared(b->options[j])) {
+        g.idx.push_back(j);
+        done[j] = 1;
+      }
+    }
+    const int n = (int)g.idx.size();
+    std::vector<Params*> pps(n);
+    std::vector<long long> pc(n + 1, 0), pf[3];
+    for (int k = 0; k < 3; ++k) pf[k].assign(n + 1, 0);
+    long long sum_chunk = 0;
+    int max_passes = 0;
+    StepLaunch sl;
+    std::memset(&sl, 0, sizeof(sl));
+    for (int q = 0; q < n; ++q) {
+      adg_state* st = states[g.idx[q]];
+      pps[q] = st->dparams;
+      const StepLaunch one = single_launch(st);
+      pc[q + 1] = pc[q] + one.total_cells;
+      for (int k = 0; k < 3; ++k) pf[k][q + 1] = pf[k][q] + one.total_faces[k];
+      sum_chunk += st->chunk;
+      sl.split_periodic = q == 0 ? one.split_periodic : sl.split_periodic & one.split_periodic;
+      if (st->cascade) sl.cascade = 1;
+      const int passes = (st->cap + st->chunk - 1) / st->chunk;
+      if (passes > max_passes) max_passes = passes;
+    }
+    void* d = nullptr;
+    const size_t bytes = sizeof(Params*) * n + sizeof(long long) * ((size_t)(n + 1) * 8 + 2);
+    if (cudaMalloc(&d, bytes) != cudaSuccess) return ADG_ERR_OOM;
+    b->mem.push_back(d);
+    Params** dpps = (Params**)d;
+    long long* dpre = (long long*)(dpps + n);
+    cudaMemcpy(dpps, pps.data(), sizeof(Params*) * n, cudaMemcpyHostToDevice);
+    cudaMemcpy(dpre, pc.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice);
+    for (int k = 0; k < 3; ++k)
+      cudaMemcpy(dpre + (size_t)(k + 1) * (n + 1), pf[k].data(), sizeof(long long) * (n + 1),
+                 cudaMemcpyHostToDevice);
+    sl.pps = dpps;
+    sl.n = n;
+    sl.pre_cells = dpre;
+    for (int k = 0; k < 3; ++k) sl.pre_faces[k] = dpre + (size_t)(k + 1) * (n + 1);
+    sl.pre_fix = dpre + (size_t)4 * (n + 1);
+    sl.pre_fb = dpre + (size_t)5 * (n + 1);
+    sl.pre_refix = dpre + (size_t)6 * (n + 1);
+    sl.pre_lim = dpre + (size_t)7 * (n + 1);          // n + 3 entries
+    sl.total_cells = pc[n];
+    for (int k = 0; k < 3; ++k) sl.total_faces[k] = pf[k][n];
+    sl.sum_chunk = sum_chunk;
+    sl.max_passes = max_passes;
+    sl.prec = g.rep->prec;
+    sl.sub32 = 3 - g.rep->sub_fp64;
+    sl.sub_f32 = g.rep->sub_f32;
+    sl.sub_reg = g.rep->sub_reg;
+    sl.flux = g.rep->flux;
+    sl.pred = effective_pred(g.rep);
+    sl.ev = nullptr;
+    g.sl = sl;
+    g.dts_off = off;
+    off += n;
+    b->groups.push_back(g);
+  }
+  if (cudaGetLastError() != cudaSuccess) return ADG_ERR_CUDA;
+  return ADG_OK;
+}
+
+// Every member's options as they are now: a changed one is uploaded, and the
+// groups are formed again where a launch description holds it (a member's
+// kernels read some options from its Params and others from the launch; the two
+// never disagree).
+int batch_options(adg_batch* b) {
+  bool same = b->options.size() == b->states.size();
+  for (size_t i = 0; i < b->states.size(); ++i) {
+    adg_state* st = b->states[i];
+    if (st->params_dirty) {
+      const int rc = upload_params(st);
+      if (rc) return rc;
+    }
+    same = same && b->options[i] == LaunchOptions(st);
+  }
+  if (same) return ADG_OK;
+  const int rc = batch_group(b);
+  if (rc) {
+    b->options.clear();               // not grouped: the next step tries again
+    return fail(b->states[0], rc, "batch: the launches of changed options");
+  }
+  return ADG_OK;
 }
 
 int batch_run(adg_batch* b, bool fixed, double cfl) {
@@ -892,90 +1023,14 @@ int adg_batch_create(adg_state* const* states, int count, void* stream, adg_batc
       return ADG_ERR_CUDA;
     }
   }
-  // groups of equal (dimension, degree, precision)
-  std::vector<int> done(count, 0);
-  int off = 0;
-  for (int i = 0; i < count; ++i) {
-    if (done[i]) continue;
-    adg_batch::Group g;
-    g.rep = states[i];
-    for (int j = i; j < count; ++j) {
-      const adg_state* a = states[i];
-      const adg_state* c = states[j];
-      if (!done[j] && a->dim == c->dim && a->N == c->N && a->prec == c->prec &&
-          a->sub_fp64 == c->sub_fp64 && a->sub_f32 == c->sub_f32 && a->sub_reg == c->sub_reg &&
-          a->flux == c->flux &&
-          effective_pred(a) == effective_pred(c)) {
-        g.idx.push_back(j);
-        done[j] = 1;
-      }
-    }
-    const int n = (int)g.idx.size();
-    std::vector<Params*> pps(n);
-    std::vector<long long> pc(n + 1, 0), pf[3];
-    for (int k = 0; k < 3; ++k) pf[k].assign(n + 1, 0);
-    long long sum_chunk = 0;
-    int max_passes = 0;
-    StepLaunch sl;
-    std::memset(&sl, 0, sizeof(sl));
-    for (int q = 0; q < n; ++q) {
-      adg_state* st = states[g.idx[q]];
-      pps[q] = st->dparams;
-      const StepLaunch one = single_launch(st);
-      pc[q + 1] = pc[q] + one.total_cells;
-      for (int k = 0; k < 3; ++k) pf[k][q + 1] = pf[k][q] + one.total_faces[k];
-      sum_chunk += st->chunk;
-      sl.split_periodic = q == 0 ? one.split_periodic : sl.split_periodic & one.split_periodic;
-      if (st->cascade) sl.cascade = 1;
-      const int passes = (st->cap + st->chunk - 1) / st->chunk;
-      if (passes > max_passes) max_passes = passes;
-    }
-    void* d = nullptr;
-    const size_t bytes = sizeof(Params*) * n + sizeof(long long) * ((size_t)(n + 1) * 8 + 2);
-    if (cudaMalloc(&d, bytes) != cudaSuccess) {
-      batch_free(b);
-      return ADG_ERR_OOM;
-    }
-    b->mem.push_back(d);
-    Params** dpps = (Params**)d;
-    long long* dpre = (long long*)(dpps + n);
-    cudaMemcpy(dpps, pps.data(), sizeof(Params*) * n, cudaMemcpyHostToDevice);
-    cudaMemcpy(dpre, pc.data(), sizeof(long long) * (n + 1), cudaMemcpyHostToDevice);
-    for (int k = 0; k < 3; ++k)
-      cudaMemcpy(dpre + (size_t)(k + 1) * (n + 1), pf[k].data(), sizeof(long long) * (n + 1),
-                 cudaMemcpyHostToDevice);
-    sl.pps = dpps;
-    sl.n = n;
-    sl.pre_cells = dpre;
-    for (int k = 0; k < 3; ++k) sl.pre_faces[k] = dpre + (size_t)(k + 1) * (n + 1);
-    sl.pre_fix = dpre + (size_t)4 * (n + 1);
-    sl.pre_fb = dpre + (size_t)5 * (n + 1);
-    sl.pre_refix = dpre + (size_t)6 * (n + 1);
-    sl.pre_lim = dpre + (size_t)7 * (n + 1);          // n + 3 entries
-    sl.total_cells = pc[n];
-    for (int k = 0; k < 3; ++k) sl.total_faces[k] = pf[k][n];
-    sl.sum_chunk = sum_chunk;
-    sl.max_passes = max_passes;
-    sl.prec = g.rep->prec;
-    sl.sub32 = 3 - g.rep->sub_fp64;
-    sl.sub_f32 = g.rep->sub_f32;
-    sl.sub_reg = g.rep->sub_reg;
-    sl.flux = g.rep->flux;
-    sl.pred = effective_pred(g.rep);
-    sl.ev = nullptr;
-    g.sl = sl;
-    g.dts_off = off;
-    off += n;
-    b->groups.push_back(g);
-  }
   if (cudaMalloc((void**)&b->d_dts, sizeof(double) * count) != cudaSuccess) {
     batch_free(b);
     return ADG_ERR_OOM;
   }
-  b->mem.push_back(b->d_dts);
-  if (cudaGetLastError() != cudaSuccess) {
+  const int rc = batch_group(b);
+  if (rc) {
     batch_free(b);
-    return ADG_ERR_CUDA;
+    return rc;
   }
   *out = b;
   return ADG_OK;
@@ -984,6 +1039,17 @@ int adg_batch_create(adg_state* const* states, int count, void* stream, adg_batc
 int adg_batch_step(adg_batch* b, const double* dts, double cfl) {
   if (!b) return ADG_ERR_ARG;
   adg_state* st0 = b->states[0];
+  if (!dts) {
+    for (adg_state* st : b->states)
+      if (!(cfl > 0.0) && !(st->cfl > 0.0))
+        return fail(st0, ADG_ERR_ARG, "cfl must be positive (argument or ADG_OPT_CFL)");
+    for (adg_state* st : b->states) {
+      const int rc = ensure_lambda(st);
+      if (rc) return rc;
+    }
+  }
+  const int ro = batch_options(b);
+  if (ro) return ro;
   if (dts) {
     // host steps in group order
     std::vector<double> ordered(b->states.size());
@@ -999,14 +1065,6 @@ int adg_batch_step(adg_batch* b, const double* dts, double cfl) {
     int rc = batch_run(b, true, 0.0);
     if (rc) return rc;
   } else {
-    for (adg_state* st : b->states)
-      if (!(cfl > 0.0) && !(st->cfl > 0.0))
-        return fail(st0, ADG_ERR_ARG, "cfl must be positive (argument or ADG_OPT_CFL)");
-    for (adg_state* st : b->states) {
-      int rc = ensure_lambda(st);
-      if (!rc && st->params_dirty) rc = upload_params(st);
-      if (rc) return rc;
-    }
     if (!(b->exec && b->graph_cfl == cfl)) {
       // one graph for the step of every group; each group's limiter passes
       // loop on the device (conditional node), sized by its troubled counts
