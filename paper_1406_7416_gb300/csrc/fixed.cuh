@@ -60,7 +60,7 @@ __device__ __forceinline__ FxOp fx_op(double m, int g) {
 __device__ __forceinline__ unsigned fx_key(double x) { return (unsigned)__double2hiint(x) * 2u; }
 
 // x on the scale of exponent field e (that of the line's largest magnitude, at
-// least FX_E_MIN), rounded toward minus infinity at 2^-58 of the scale.
+// least FX_E_MIN), cut toward zero at 2^-58 of the scale.
 __device__ __forceinline__ FxVal fx_val(double x, unsigned e) {
   const int hi = __double2hiint(x);
   const unsigned lo = (unsigned)__double2loint(x);
@@ -72,13 +72,24 @@ __device__ __forceinline__ FxVal fx_val(double x, unsigned e) {
   asm("{.reg .b64 a; mov.b64 a, {%1, %2}; shr.u64 %0, a, %3;}"
       : "=l"(f)
       : "r"(lo << 11), "r"(__funnelshift_l(lo, mh, 11)), "r"(s));
-  const unsigned sg = (unsigned)(hi >> 31);          // the sign as a complement
-  const unsigned fl = (unsigned)f ^ sg, fh = (unsigned)(f >> 32) ^ sg;
+  const unsigned sg = (unsigned)(hi >> 31);          // all ones: negative
+  unsigned fl, fh;
+  asm("{sub.cc.u32 %0, %2, %4; subc.u32 %1, %3, %4;}"
+      : "=r"(fl), "=r"(fh)
+      : "r"((unsigned)f ^ sg), "r"((unsigned)(f >> 32) ^ sg), "r"(sg));
   FxVal o;
   o.l = (int)fl;
   o.h = (int)(fh + (fl >> 31));
   return o;
 }
+
+// A dot product in units of 2^64: (r 2^32 + f) 2^-32, |r| < 2^58.
+struct FxSum {
+  long long r;
+  unsigned f;
+  // cut toward zero
+  __device__ __forceinline__ long long cut() const { return r + (long long)(r < 0 && f != 0u); }
+};
 
 // Accumulator of a dot product: entries times values, without the low x low
 // products (below 2^-57 of the row sum times the largest element).
@@ -90,18 +101,22 @@ struct FxAcc {
     hl = fx_mad(x.h, m.l, hl);
     hl = fx_mad(x.l, m.h, hl);
   }
-  // the sum in units of 2^64 (below 2^58)
-  __device__ __forceinline__ long long sum() const { return fx_mad((int)(hl >> 32), 1, hh); }
+  __device__ __forceinline__ FxSum sum() const { return {fx_mad((int)(hl >> 32), 1, hh), (unsigned)hl}; }
 };
 
-// The value R 2^(b - 1085) as a double, rounded to nearest (b: an exponent
-// field, at least 70 and at most 2040).  A dot product of a line with exponent
-// field e by an operator with scale exponent g has b = e + g + 5.
-__device__ __forceinline__ double fx_double(long long R, int b) {
+// The sum R, cut toward zero to whole units, times 2^(b - 1085) as a double,
+// rounded to nearest (b: an exponent field, at least 70 and at most 2040).
+// Odd in R, and zero where the whole units are.  A dot product of a line with
+// exponent field e by an operator with scale exponent g has b = e + g + 5.
+__device__ __forceinline__ double fx_double(FxSum R, int b) {
   int rl, rh;
-  asm("mov.b64 {%0, %1}, %2;" : "=r"(rl), "=r"(rh) : "l"(R));
+  asm("mov.b64 {%0, %1}, %2;" : "=r"(rl), "=r"(rh) : "l"(R.r));
   const unsigned s = (unsigned)(rh >> 31);
-  const unsigned al = (unsigned)rl ^ s, ah = (unsigned)rh ^ s;
+  // whole units of |R|: of a negative one the complement of r, one more if f = 0
+  unsigned al, ah;
+  asm("{.reg .u32 d; add.cc.u32 d, %4, 0xffffffff; addc.cc.u32 %0, %2, 0; addc.u32 %1, %3, 0;}"
+      : "=r"(al), "=r"(ah)
+      : "r"((unsigned)rl ^ s), "r"((unsigned)rh ^ s), "r"(R.f == 0u ? s : 0u));
   const bool z = ah == 0;
   const unsigned x = z ? al : ah, y = z ? 0u : al;
   const int lz = __clz((int)x);
@@ -113,7 +128,7 @@ __device__ __forceinline__ double fx_double(long long R, int b) {
   asm("{.reg .u32 d; add.cc.u32 d, %2, %2; addc.cc.u32 %0, %3, 0; addc.u32 %1, %4, %5;}"
       : "=r"(ol), "=r"(oh)
       : "r"(nl << 21), "r"(bl), "r"(bh), "r"(eb));
-  return __hiloint2double((int)(oh | (s & 0x80000000u)), (int)ol);
+  return __hiloint2double(x == 0u ? 0 : (int)(oh | (s & 0x80000000u)), (int)ol);
 }
 
 // ROWS outputs of an operator on the line x: out(a, sum_j m[a n + j] x[j]) for

@@ -788,12 +788,12 @@ __global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
             acc.add(x, row[k][j]);
           }
         }
-        Sv[v] = e < FX_E_MIN ? 0 : acc.sum();
+        Sv[v] = e < FX_E_MIN ? 0 : acc.sum().cut();
         es[v] = e;
       }
     };
     // u - (R as a double), R on the scale of a dot product of S by Ktau
-    auto close = [&](double u0, long long R, unsigned e) {
+    auto close = [&](double u0, FxSum R, unsigned e) {
       const int bf = (int)e + gD + gK + 6;
       double x = fx_double(R, bf);
       if (bf < 70) x = 0.0;

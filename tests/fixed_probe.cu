@@ -1,0 +1,57 @@
+// Test probe: fx_apply of csrc/fixed.cuh on lines and operators from the host.
+#include <cuda_runtime.h>
+
+#include "../paper_1406_7416_gb300/csrc/fixed.cuh"
+
+namespace {
+
+using namespace adg;
+
+// out[line][n] = M x[line] for an n x n operator
+template <int n>
+__global__ void products(const double* M, const double* x, long long lines, double* out) {
+  __shared__ FxOp m[n * n];
+  __shared__ int g;
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int a = 0; a < n; ++a) {
+      double r = 0.0;
+      for (int j = 0; j < n; ++j) r += fabs(M[a * n + j]);
+      s = r > s ? r : s;
+    }
+    g = fx_scale(s);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n * n; i += blockDim.x) m[i] = fx_op(M[i], g);
+  __syncthreads();
+  for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < lines;
+       l += (long long)gridDim.x * blockDim.x) {
+    double v[n];
+#pragma unroll
+    for (int j = 0; j < n; ++j) v[j] = x[l * n + j];
+    fx_apply<n, n>(v, m, g, [&](int a, double y) { out[l * n + a] = y; });
+  }
+}
+
+template <int n>
+int run(int want, const double* M, const double* x, long long lines, double* out) {
+  if (want != n) {
+    if constexpr (n < 10) return run<n + 1>(want, M, x, lines, out);
+    return -1;
+  }
+  double* d = nullptr;
+  if (cudaMalloc(&d, sizeof(double) * (n * n + 2 * lines * n)) != cudaSuccess) return -2;
+  double *dx = d + n * n, *dout = dx + lines * n;
+  cudaMemcpy(d, M, sizeof(double) * n * n, cudaMemcpyHostToDevice);
+  cudaMemcpy(dx, x, sizeof(double) * lines * n, cudaMemcpyHostToDevice);
+  products<n><<<64, 128>>>(d, dx, lines, dout);
+  const cudaError_t e = cudaMemcpy(out, dout, sizeof(double) * lines * n, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e == cudaSuccess ? 0 : -3;
+}
+
+}  // namespace
+
+extern "C" int fixed_products(int n, const double* M, const double* x, long long lines, double* out) {
+  return run<1>(n, M, x, lines, out);
+}

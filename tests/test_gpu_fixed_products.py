@@ -1,0 +1,90 @@
+"""GPU: products of lines of doubles with an operator on the integer pipes (fx_apply of
+csrc/fixed.cuh), called by themselves through tests/fixed_probe.cu, against exact rational
+arithmetic."""
+import ctypes
+import os
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+from oracle.basis import Basis
+from paper_1406_7416_gb300 import build_lib
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def products(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("probe") / "fixed_probe.so")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "fixed_probe.cu")
+    subprocess.run([build_lib._nvcc()] + build_lib.NVCC_FLAGS + ["-shared", src, "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    ptr = np.ctypeslib.ndpointer(np.float64, flags="C")
+    lib.fixed_products.argtypes = [ctypes.c_int, ptr, ptr, ctypes.c_longlong, ptr]
+
+    def call(M, x):
+        M, x = np.ascontiguousarray(M, float), np.ascontiguousarray(x, float)
+        out = np.empty_like(x)
+        assert lib.fixed_products(M.shape[0], M, x, x.shape[0], out) == 0
+        return out
+    return call
+
+
+def _exact(M, x):
+    """The exact products as Fractions."""
+    F = [[Fraction(float(v)) for v in row] for row in M]
+    return [[sum(m * Fraction(float(v)) for m, v in zip(row, line)) for row in F] for line in x]
+
+
+def _lines(n, count, seed):
+    rng = np.random.default_rng(seed)
+    return rng.uniform(-1, 1, (count, n)) * 2.0 ** rng.integers(-4, 1, (count, n)) * \
+        2.0 ** rng.integers(-60, 60, (count, 1))
+
+
+@pytest.mark.parametrize("n", range(2, 11))
+def test_cancelling_products_are_zero(products, n):
+    """An antisymmetric row on a line of equal elements, and rows of a line of zeros, give zero."""
+    rng = np.random.default_rng(n)
+    half = rng.uniform(0.1, 3.0, (n, n // 2))
+    mid = np.zeros((n, n % 2))
+    M = np.concatenate([half, mid, -half[:, ::-1]], axis=1)
+    x = np.repeat(_lines(1, 500, n), n, axis=1)
+    x[::7] = 0.0
+    x[1::7] = 3.0
+    x[2::7] = -0.25
+    assert np.array_equal(products(M, x), np.zeros_like(x))
+
+
+@pytest.mark.parametrize("n", range(1, 11))
+def test_products_are_odd(products, n):
+    """f(-x) = -f(x), bit for bit, small whole numbers (whose products end in zero bits) included."""
+    rng = np.random.default_rng(n)
+    M = rng.uniform(-2, 2, (n, n))
+    x = _lines(n, 2000, 3 * n)
+    x[::3] = rng.integers(-4, 5, x[::3].shape)
+    y = products(M, x)
+    assert np.array_equal(products(M, -x), -y)
+    assert np.abs(y).max() > 0
+
+
+@pytest.mark.parametrize("n", range(1, 11))
+def test_products_against_exact_ones(products, n):
+    """Error of each output in units of s m, s the operator's largest row sum and m the line's
+    largest magnitude: elements cut at 2^-58 m, entries rounded at 2^-62 s, the n products of low
+    halves left out (each below 2^-57), the sum cut at 2^-55, and the result rounded to 53 bits."""
+    M = Basis(n - 1).D if n > 1 else np.array([[1.7]])
+    x = _lines(n, 150, 7 * n)
+    y = products(M, x)
+    s, m = np.abs(M).sum(axis=1).max(), np.abs(x).max(axis=1)
+    bar = Fraction(1, 2 ** 58) + n * Fraction(1, 2 ** 62) + n * Fraction(1, 2 ** 57) + \
+        Fraction(1, 2 ** 55) + Fraction(1, 2 ** 53)
+    worst = 0.0
+    for l, row in enumerate(_exact(M, x)):
+        for a, v in enumerate(row):
+            err = abs(Fraction(float(y[l, a])) - v)
+            assert err <= bar * Fraction(float(s)) * Fraction(float(m[l])), (l, a, float(err))
+            worst = max(worst, float(err) / (s * m[l]))
+    print(n, worst)
