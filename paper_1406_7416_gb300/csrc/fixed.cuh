@@ -30,10 +30,12 @@ struct FxVal {
   int h, l;
 };
 
-// Exponent fields (of doubles) between which a line is worked on: a line whose
-// largest magnitude is below 2^-959 counts as zero, one from 2^977 on (or with
-// an infinity or a NaN) gives NaN.
+// Exponent fields (of doubles) between which a line is worked on in integers;
+// lines below 2^-959, from 2^977 on, or with an infinity or a NaN take the
+// FP64 pipe.
 constexpr unsigned FX_E_MIN = 64, FX_E_MAX = 2000;
+// ... and those of results (fx_double)
+constexpr int FX_B_MIN = 70, FX_B_MAX = 2040;
 
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
   long long d;
@@ -42,9 +44,11 @@ __device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
 }
 
 // Scale exponent g of an operator whose largest row sum of magnitudes is s
-// (positive and finite): s < 2^(g - 1), so every entry is below 2^62.
+// (positive): s < 2^(g - 1), so every entry is below 2^62.  (An overflown s:
+// out of every range, so that the FP64 pipe takes the lines.)
 __device__ __forceinline__ int fx_scale(double s) {
-  return ((__double2hiint(s) >> 20) & 0x7ff) - 1023 + 2;
+  const int e = (__double2hiint(s) >> 20) & 0x7ff;
+  return e == 0x7ff ? 1 << 16 : e - 1023 + 2;
 }
 
 // Entry m of an operator with scale exponent g.
@@ -87,8 +91,6 @@ __device__ __forceinline__ FxVal fx_val(double x, unsigned e) {
 struct FxSum {
   long long r;
   unsigned f;
-  // cut toward zero
-  __device__ __forceinline__ long long cut() const { return r + (long long)(r < 0 && f != 0u); }
 };
 
 // Accumulator of a dot product: entries times values, without the low x low
@@ -105,7 +107,7 @@ struct FxAcc {
 };
 
 // The sum R, cut toward zero to whole units, times 2^(b - 1085) as a double,
-// rounded to nearest (b: an exponent field, at least 70 and at most 2040).
+// rounded to nearest (b: an exponent field in FX_B_MIN .. FX_B_MAX).
 // Odd in R, and zero where the whole units are.  A dot product of a line with
 // exponent field e by an operator with scale exponent g has b = e + g + 5.
 __device__ __forceinline__ double fx_double(FxSum R, int b) {
@@ -131,18 +133,47 @@ __device__ __forceinline__ double fx_double(FxSum R, int b) {
   return __hiloint2double(x == 0u ? 0 : (int)(oh | (s & 0x80000000u)), (int)ol);
 }
 
+// The same product on the FP64 pipe: rows of doubles, times c.  Out of line: the
+// lines outside the range are rare, and their code would cost the others registers.
+__device__ __noinline__ static double fx_dot(const double* m, const double* x, int n) {
+  double acc = 0.0;
+  for (int j = 0; j < n; ++j) acc = fma(m[j], x[j], acc);
+  return acc;
+}
+struct FxRows {
+  const double* m;
+  double c;
+  template <int n>
+  __device__ __forceinline__ double row(const double* x, int a) const {
+    return c * fx_dot(m + a * n, x, n);
+  }
+};
+
+// Rows that are the row sums of an operator of L columns, on "lines" of one.
+template <int L>
+struct FxSums {
+  const double* m;
+  template <int n>
+  __device__ __forceinline__ double row(const double* x, int a) const {
+    double s = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < L; ++j) s += m[a * L + j];
+    return s * x[0];
+  }
+};
+
 // ROWS outputs of an operator on the line x: out(a, sum_j m[a n + j] x[j]) for
-// a < ROWS, m of scale exponent g.  Lines out of the range are settled by a
-// branch: zero, or NaN in every output (as a line with a NaN or an infinity
-// has in FP64, up to the sign of an infinity).
-template <int n, int ROWS, typename Out>
-__device__ __forceinline__ void fx_apply(const double* x, const FxOp* __restrict__ m, int g, Out out) {
+// a < ROWS, m of scale exponent g, `rows` its rows in FP64.  Lines out of the
+// range take the FP64 pipe.
+template <int n, int ROWS, typename Rows, typename Out>
+__device__ __forceinline__ void fx_apply(const double* x, const FxOp* __restrict__ m, int g, Rows rows,
+                                         Out out) {
   unsigned key = 0;
 #pragma unroll
   for (int j = 0; j < n; ++j) key = max(key, fx_key(x[j]));
   const unsigned e = key >> 21;
   const int b = (int)e + g + 5;
-  if (e >= FX_E_MIN && e < FX_E_MAX && b >= 70 && b <= 2040) {
+  if (e >= FX_E_MIN && e < FX_E_MAX && b >= FX_B_MIN && b <= FX_B_MAX) {
     FxVal f[n];
 #pragma unroll
     for (int j = 0; j < n; ++j) f[j] = fx_val(x[j], e);
@@ -155,9 +186,15 @@ __device__ __forceinline__ void fx_apply(const double* x, const FxOp* __restrict
       out(a, fx_double(acc.sum(), b));
     }
   } else {
-    const double fill = (e < FX_E_MIN || b < 70) ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+    unsigned low = 0;                                   // (a line of zeros, a flow at rest, has no sums)
+#pragma unroll
+    for (int j = 0; j < n; ++j) low |= (unsigned)__double2loint(x[j]);
+    const bool zero = (key | low) == 0;
+    double y[n];
+#pragma unroll
+    for (int j = 0; j < n; ++j) y[j] = x[j];
 #pragma unroll 1
-    for (int a = 0; a < ROWS; ++a) out(a, fill);
+    for (int a = 0; a < ROWS; ++a) out(a, zero ? 0.0 : rows.template row<n>(y, a));
   }
 }
 

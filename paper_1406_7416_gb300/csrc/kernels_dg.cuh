@@ -147,10 +147,13 @@ __device__ __forceinline__ void flux_fx(const double* __restrict__ q, double* __
 }
 
 // Derivative phase, F_k <- (c_k D) x_k F_k in place for every axis: one thread
-// per line of n nodes (cD[k n n ..] is c_k D with scale exponent gD[k]).  NL
-// lines per variable (those of all time nodes, or of time node 0).
+// per line of n nodes (cD[k n n ..] is c_k D with scale exponent gD[k]; coef and
+// Dm its factors).  NL lines per variable (those of all time nodes, or of time
+// node 0).
 template <int D, int n, int NL>
-__device__ __forceinline__ void deriv_fx(double* F, const FxOp* cD, const int* gD, int tid, int nth) {
+__device__ __forceinline__ void deriv_fx(double* F, const FxOp* cD, const int* gD,
+                                         const double* __restrict__ coef, const double* __restrict__ Dm,
+                                         int tid, int nth) {
   constexpr int NV = D + 2, NST = ipow(n, D + 1);
   for (int e = tid; e < D * NV * NL; e += nth) {
     const int kv = e / NL, r = e - kv * NL;
@@ -160,14 +163,14 @@ __device__ __forceinline__ void deriv_fx(double* F, const FxOp* cD, const int* g
     double x[n];
 #pragma unroll
     for (int j = 0; j < n; ++j) x[j] = f[j * st];
-    fx_apply<n, n>(x, cD + k * (n * n), gD[k], [&](int a, double y) { f[a * st] = y; });
+    fx_apply<n, n>(x, cD + k * (n * n), gD[k], FxRows{Dm, coef[k]}, [&](int a, double y) { f[a * st] = y; });
   }
 }
 
 // Time phase, q <- u - Ktau S with S = sum_k of the derivative phase's F_k.
 template <int D, int n>
 __device__ __forceinline__ void time_fx(const double* F, double* q, const double* u, const FxOp* Kt,
-                                        int gK, int tid, int nth) {
+                                        int gK, const double* __restrict__ Ktd, int tid, int nth) {
   constexpr int NV = D + 2, ND = ipow(n, D), NST = ipow(n, D + 1);
   for (int e = tid; e < NV * ND; e += nth) {
     const int v = e / ND, i = e - v * ND;
@@ -181,7 +184,7 @@ __device__ __forceinline__ void time_fx(const double* F, double* q, const double
     }
     const double u0 = u[e];
     double* qv = q + v * NST + i;
-    fx_apply<n, n>(S, Kt, gK, [&](int m, double y) { qv[m * ND] = u0 - y; });
+    fx_apply<n, n>(S, Kt, gK, FxRows{Ktd, 1.0}, [&](int m, double y) { qv[m * ND] = u0 - y; });
   }
 }
 
@@ -522,7 +525,7 @@ __device__ __forceinline__ void apply_pass_fx(const double* in, double* out, con
       double x[NI];
 #pragma unroll
       for (int j = 0; j < NI; ++j) x[j] = src[j * S];
-      fx_apply<NI, NO>(x, M.x, M.g, [&](int a, double y) { dst[a * S] = y; });
+      fx_apply<NI, NO>(x, M.x, M.g, FxRows{M.d, 1.0}, [&](int a, double y) { dst[a * S] = y; });
     }
   }
 }
@@ -743,7 +746,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
       // q_m = u - kappa_m S with kappa = Ktau 1
       flux_fx<D, n>(u, F, gm1, ND, ND, tid, nth);
       __syncthreads();
-      deriv_fx<D, n, ND / n>(F, cD, gD, tid, nth);
+      deriv_fx<D, n, ND / n>(F, cD, gD, p.b.coef, o->D, tid, nth);
       __syncthreads();
       for (int e = tid; e < NV * ND; e += nth) {
         const int v = e / ND, i = e - v * ND;
@@ -752,7 +755,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
         for (int k = 1; k < D; ++k) S += F[(k * NV + v) * NST + i];
         const double u0 = u[e];
         double* qv = q + v * NST + i;
-        fx_apply<1, n>(&S, kapx, gK, [&](int m, double y) { qv[m * ND] = u0 - y; });
+        fx_apply<1, n>(&S, kapx, gK, FxSums<n>{o->Kt}, [&](int m, double y) { qv[m * ND] = u0 - y; });
       }
       it0 = 1;
     }
@@ -760,9 +763,9 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
     for (int it = it0; it < p.iters; ++it) {
       flux_fx<D, n>(q, F, gm1, NST, NST, tid, nth);
       __syncthreads();
-      deriv_fx<D, n, NST / n>(F, cD, gD, tid, nth);
+      deriv_fx<D, n, NST / n>(F, cD, gD, p.b.coef, o->D, tid, nth);
       __syncthreads();
-      time_fx<D, n>(F, q, u, Ktx, gK, tid, nth);
+      time_fx<D, n>(F, q, u, Ktx, gK, o->Kt, tid, nth);
       __syncthreads();
     }
     if (split) {
@@ -834,7 +837,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
         double x[n];
 #pragma unroll
         for (int m = 0; m < n; ++m) x[m] = F[kv * NST + i + m * ND];
-        fx_apply<n, 1>(x, wx, gw, [&](int, double y) { fbar[e] = y; });
+        fx_apply<n, 1>(x, wx, gw, FxRows{w, 1.0}, [&](int, double y) { fbar[e] = y; });
       }
       __syncthreads();
     }
@@ -847,7 +850,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
       double x[n];
 #pragma unroll
       for (int j = 0; j < n; ++j) x[j] = f[j * st];
-      fx_apply<n, n>(x, cM + k * (n * n), gM[k], [&](int a, double y) { f[a * st] = y; });
+      fx_apply<n, n>(x, cM + k * (n * n), gM[k], FxRows{o->Mvol, p.b.coef[k]}, [&](int a, double y) { f[a * st] = y; });
     }
     // space-time traces on the faces, trace[cell][k][side][v][ts + NF * m], by
     // lines: the n nodes of a line along axis k give both faces normal to k, and
@@ -861,7 +864,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
 #pragma unroll
         for (int j = 0; j < n; ++j) x[j] = f[j * st];
         double* t = tr + (2 * k) * (NV * NT) + vr;
-        fx_apply<n, 2>(x, phx, gph, [&](int side, double y) { t[side * (NV * NT)] = y; });
+        fx_apply<n, 2>(x, phx, gph, FxRows{ph0, 1.0}, [&](int side, double y) { t[side * (NV * NT)] = y; });
       }
     __syncthreads();
     double* Uo = p.b.U[1 - p.cur] + cell * (NV * ND);

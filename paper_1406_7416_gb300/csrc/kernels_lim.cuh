@@ -661,6 +661,52 @@ __global__ void __launch_bounds__(256) k_lim_predict(Batch bt, int pass, int n32
   }
 }
 
+// The FP64 subcell predictor of a warp's subcells with its contractions on the
+// FP64 pipe (lanes, lines and operators as in k_lim_predict_i): x[v] the lane's
+// reconstruction on entry, x[m NV + v] its three time nodes on return.  For
+// magnitudes outside the fixed-point range, which are rare: out of line, rolled.
+template <int D>
+__device__ __noinline__ void sub_predict_fp64(double* x, const double* ck, double gm1, const Ops* o, int sx,
+                                              int sy, int sz, int a, int b, int c) {
+  constexpr int NV = D + 2;
+  constexpr unsigned FULL = 0xffffffffu;
+  double u[NV], S[3][NV];
+  for (int v = 0; v < NV; ++v) {
+    u[v] = x[v];
+    x[NV + v] = x[2 * NV + v] = u[v];
+  }
+#pragma unroll 1
+  for (int it = 0; it < 3; ++it) {
+#pragma unroll 1
+    for (int m = 0; m < 3; ++m) {
+      double Q[NV], F[D][D + 2];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Q[v] = x[m * NV + v];
+      euler_fluxes_sym<D>(Q, gm1, F);
+#pragma unroll 1
+      for (int v = 0; v < NV; ++v) {
+        double s = 0.0;
+#pragma unroll 1
+        for (int k = 0; k < D; ++k) {
+          const int base = k == 0 ? sx : (k == 1 ? sy : sz), st = k == 0 ? 1 : (k == 1 ? 3 : 9);
+          const double* row = o->D3 + 3 * (k == 0 ? a : (k == 1 ? b : c));
+          double t = 0.0;
+          for (int j = 0; j < 3; ++j) t = fma(row[j], __shfl_sync(FULL, F[k][v], base + j * st), t);
+          s = fma(ck[k], t, s);
+        }
+        S[m][v] = s;
+      }
+    }
+#pragma unroll 1
+    for (int m = 0; m < 3; ++m)
+      for (int v = 0; v < NV; ++v) {
+        double t = 0.0;
+        for (int j = 0; j < 3; ++j) t = fma(o->Kt3[3 * m + j], S[j][v], t);
+        x[m * NV + v] = u[v] - t;
+      }
+  }
+}
+
 // L4 in FP64: the subcell predictor in registers with its contractions on the
 // integer pipes (fixed.cuh).  What bounds the FP64 limiter is the FP64 pipe (two
 // operations per clock and multiprocessor): of the 22 FP64 operations that a
@@ -755,6 +801,13 @@ __global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
     double u[NV], q[3][NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) u[v] = (double)W[((j0 * NV + v) * NED + sc) * ND3 + node];
+    // outside the range of the fixed-point products: fluxes by FX_E_MAX, results by
+    // FX_B_MIN and FX_B_MAX, and fluxes of a variable below 2^-900 (not zero), which
+    // may be below FX_E_MIN
+    bool far = false;
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+      far = far || (fx_key(u[v]) < ((1023u - 900u) << 21) && (fx_key(u[v]) | (unsigned)__double2loint(u[v])) != 0u);
     // S = sum_k c_k D x_k F_k(Q) at this node: Sv[v] 2^64 on the scale es[v]
     auto space_term = [&](const double* Q, long long* Sv, unsigned* es) {
       double F[D][D + 2];
@@ -788,17 +841,16 @@ __global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
             acc.add(x, row[k][j]);
           }
         }
-        Sv[v] = e < FX_E_MIN ? 0 : acc.sum().cut();
-        es[v] = e;
+        Sv[v] = acc.sum().r;
+        es[v] = ec;
       }
     };
     // u - (R as a double), R on the scale of a dot product of S by Ktau
     auto close = [&](double u0, FxSum R, unsigned e) {
       const int bf = (int)e + gD + gK + 6;
-      double x = fx_double(R, bf);
-      if (bf < 70) x = 0.0;
-      if (e >= FX_E_MAX || bf > 2040) x = __longlong_as_double(0x7ff8000000000000LL);
-      return u0 - x;
+      far = far || e >= FX_E_MAX || bf > FX_B_MAX || (bf < FX_B_MIN && R.r != 0);
+      const double x = fx_double(R, bf);
+      return u0 - (bf < FX_B_MIN ? 0.0 : x);
     };
     {
       long long S[NV];
@@ -813,7 +865,7 @@ __global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
         for (int m = 0; m < 3; ++m) {
           FxAcc acc;
           acc.add(x, kap[m]);
-          q[m][v] = close(u[v], acc.sum(), max(es[v], FX_E_MIN));
+          q[m][v] = close(u[v], acc.sum(), es[v]);
         }
       }
     }
@@ -825,11 +877,11 @@ __global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
       for (int m = 0; m < 3; ++m) space_term(q[m], S[m], es[m]);
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
-        const unsigned e = max(max(es[0][v], es[1][v]), max(es[2][v], FX_E_MIN));
+        const unsigned e = max(max(es[0][v], es[1][v]), es[2][v]);
         FxVal x[3];
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-          const unsigned sh = e - max(es[m][v], FX_E_MIN);
+          const unsigned sh = e - es[m][v];
           const long long s = S[m][v] >> (sh < 63u ? sh : 63u);
           x[m].l = (int)s;
           x[m].h = (int)((s - x[m].l) >> 32);
@@ -842,6 +894,18 @@ __global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
           q[m][v] = close(u[v], acc.sum(), e);
         }
       }
+    }
+    if (__any_sync(FULL, far)) {
+      double x[3 * NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) x[v] = u[v];
+      sub_predict_fp64<D>(x, p.b.coef + 3, gm1, o, sx, sy, sz, a, b, c);
+      const bool own = D == 3 || (__ballot_sync(FULL, far) >> (9 * grp) & 0x1ffu) != 0u;
+#pragma unroll
+      for (int m = 0; m < 3; ++m)
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+          if (own) q[m][v] = x[m * NV + v];
     }
     if (live) {
       double* dst = p.b.qsub + ((size_t)j0 * NED + sc) * (size_t)(NV * NST3);
@@ -1730,8 +1794,8 @@ __global__ void __launch_bounds__(128) k_lim_flux_d(Batch bt, int pass) {
         const double* a = qL + v * NST3;
         const double* b = qR + v * NST3;
         const double xa[3] = {a[0], a[stk], a[2 * stk]}, xb[3] = {b[0], b[stk], b[2 * stk]};
-        fx_apply<3, 1>(xa, ph[0], g, [&](int, double y) { QL[v] = y; });
-        fx_apply<3, 1>(xb, ph[1], g, [&](int, double y) { QR[v] = y; });
+        fx_apply<3, 1>(xa, ph[0], g, FxRows{o->phi13, 1.0}, [&](int, double y) { QL[v] = y; });
+        fx_apply<3, 1>(xb, ph[1], g, FxRows{o->phi03, 1.0}, [&](int, double y) { QR[v] = y; });
       }
       if (wall < 0) {
 #pragma unroll

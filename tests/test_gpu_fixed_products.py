@@ -88,3 +88,29 @@ def test_products_against_exact_ones(products, n):
             assert err <= bar * Fraction(float(s)) * Fraction(float(m[l])), (l, a, float(err))
             worst = max(worst, float(err) / (s * m[l]))
     print(n, worst)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 6, 9, 10])
+@pytest.mark.parametrize("e", [-1060, -1000, -962, -958, 974, 980, 1010])
+def test_lines_at_the_ends_of_the_range(products, n, e):
+    """Lines below 2^-959 (subnormals too) and from 2^977 on: every product rounds at 2^-53 of
+    its terms, or at the last place of a subnormal."""
+    M = Basis(n - 1).D if n > 1 else np.array([[1.7]])
+    x = np.ldexp(_lines(n, 40, n), 0)
+    x = np.ldexp(x / np.abs(x).max(axis=1, keepdims=True), e)
+    x[3] = 0.0
+    y = products(M, x)
+    s, m = np.abs(M).sum(axis=1).max(), np.abs(x).max(axis=1)
+    for l, row in enumerate(_exact(M, x)):
+        for a, v in enumerate(row):
+            bar = (n + 1) * Fraction(float(s)) * Fraction(float(m[l])) / 2 ** 53 + n * Fraction(1, 2 ** 1074)
+            assert abs(Fraction(float(y[l, a])) - v) <= bar, (l, a)
+
+
+@pytest.mark.parametrize("n", [1, 2, 5])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_lines_with_a_nan_or_an_infinity(products, n, bad):
+    x = np.ones((6, n))
+    x[2, n // 2] = bad
+    y = products(np.full((n, n), 1.5), x)
+    assert not np.isfinite(y[2]).any() and np.isfinite(np.delete(y, 2, axis=0)).all()
