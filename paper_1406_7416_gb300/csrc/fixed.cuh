@@ -133,19 +133,28 @@ __device__ __forceinline__ double fx_double(FxSum R, int b) {
   return __hiloint2double(x == 0u ? 0 : (int)(oh | (s & 0x80000000u)), (int)ol);
 }
 
-// The same product on the FP64 pipe: rows of doubles, times c.  Out of line: the
-// lines outside the range are rare, and their code would cost the others registers.
-__device__ __noinline__ static double fx_dot(const double* m, const double* x, int n) {
-  double acc = 0.0;
-  for (int j = 0; j < n; ++j) acc = fma(m[j], x[j], acc);
-  return acc;
+// Rows of doubles, times c: y(a) = c sum_j m[a n + j] x[j] on the FP64 pipe.
+// Out of line: the lines that take it are few, and its code would cost the
+// others registers.
+template <int n>
+__device__ __noinline__ void fx_rows(const double* m, double c, int rows, const double* x, double* y) {
+  double v[n];
+#pragma unroll
+  for (int j = 0; j < n; ++j) v[j] = x[j];
+#pragma unroll 1
+  for (int a = 0; a < rows; ++a) {
+    double acc = 0.0;
+#pragma unroll
+    for (int j = 0; j < n; ++j) acc = fma(m[a * n + j], v[j], acc);
+    y[a] = c * acc;
+  }
 }
 struct FxRows {
   const double* m;
   double c;
-  template <int n>
-  __device__ __forceinline__ double row(const double* x, int a) const {
-    return c * fx_dot(m + a * n, x, n);
+  template <int n, int ROWS>
+  __device__ __forceinline__ void apply(const double* x, double* y) const {
+    fx_rows<n>(m, c, ROWS, x, y);
   }
 };
 
@@ -153,27 +162,44 @@ struct FxRows {
 template <int L>
 struct FxSums {
   const double* m;
-  template <int n>
-  __device__ __forceinline__ double row(const double* x, int a) const {
-    double s = 0.0;
+  template <int n, int ROWS>
+  __device__ __forceinline__ void apply(const double* x, double* y) const {
 #pragma unroll 1
-    for (int j = 0; j < L; ++j) s += m[a * L + j];
-    return s * x[0];
+    for (int a = 0; a < ROWS; ++a) {
+      double s = 0.0;
+#pragma unroll 1
+      for (int j = 0; j < L; ++j) s += m[a * L + j];
+      y[a] = s * x[0];
+    }
   }
 };
 
 // ROWS outputs of an operator on the line x: out(a, sum_j m[a n + j] x[j]) for
-// a < ROWS, m of scale exponent g, `rows` its rows in FP64.  Lines out of the
-// range take the FP64 pipe.
-template <int n, int ROWS, typename Rows, typename Out>
+// a < ROWS, m of scale exponent g, `rows` its rows in FP64.
+//
+// Two kinds of lines take the FP64 pipe: those out of the range, and steep ones.
+// The integers hold every element to 2^-58 of the largest, and a row may give the
+// largest next to no weight: the far side of a jump, or a spike in the middle of a
+// differentiated line.  Its result then has only the small elements' bits.  Each
+// row's large weights are those of the nodes around its own, so with one of every
+// two neighbours (of three, one of the outer ones too) within 2^-5 of the largest
+// the error stays that of the FMA chain; other lines (the cells a shock runs
+// through) are left to it.  EVEN: no need to look (every weight of the operator is
+// at least 1/32 of its row, or as its caller says).
+template <int n, int ROWS, bool EVEN, typename Rows, typename Out>
 __device__ __forceinline__ void fx_apply(const double* x, const FxOp* __restrict__ m, int g, Rows rows,
                                          Out out) {
-  unsigned key = 0;
+  unsigned key = fx_key(x[0]), low = ~0u;
 #pragma unroll
-  for (int j = 0; j < n; ++j) key = max(key, fx_key(x[j]));
+  for (int j = 1; j < n; ++j) {
+    if (!EVEN && n > 2) low = min(low, max(fx_key(x[j - 1]), fx_key(x[j])));
+    key = max(key, fx_key(x[j]));
+  }
+  if (!EVEN && n == 3) low = min(low, max(fx_key(x[0]), fx_key(x[n - 1])));
   const unsigned e = key >> 21;
   const int b = (int)e + g + 5;
-  if (e >= FX_E_MIN && e < FX_E_MAX && b >= FX_B_MIN && b <= FX_B_MAX) {
+  const bool steep = !EVEN && n > 2 && (low >> 21) + 5u < e;
+  if (e >= FX_E_MIN && e < FX_E_MAX && b >= FX_B_MIN && b <= FX_B_MAX && !steep) {
     FxVal f[n];
 #pragma unroll
     for (int j = 0; j < n; ++j) f[j] = fx_val(x[j], e);
@@ -186,15 +212,15 @@ __device__ __forceinline__ void fx_apply(const double* x, const FxOp* __restrict
       out(a, fx_double(acc.sum(), b));
     }
   } else {
-    unsigned low = 0;                                   // (a line of zeros, a flow at rest, has no sums)
+    unsigned any = key;                                 // (a line of zeros, a flow at rest, has no sums)
 #pragma unroll
-    for (int j = 0; j < n; ++j) low |= (unsigned)__double2loint(x[j]);
-    const bool zero = (key | low) == 0;
-    double y[n];
+    for (int j = 0; j < n; ++j) any |= (unsigned)__double2loint(x[j]);
+    double v[n], y[ROWS];
 #pragma unroll
-    for (int j = 0; j < n; ++j) y[j] = x[j];
+    for (int j = 0; j < n; ++j) v[j] = x[j];
+    if (any) rows.template apply<n, ROWS>(v, y);
 #pragma unroll 1
-    for (int a = 0; a < ROWS; ++a) out(a, zero ? 0.0 : rows.template row<n>(y, a));
+    for (int a = 0; a < ROWS; ++a) out(a, any ? y[a] : 0.0);
   }
 }
 

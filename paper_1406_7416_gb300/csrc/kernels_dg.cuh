@@ -163,7 +163,7 @@ __device__ __forceinline__ void deriv_fx(double* F, const FxOp* cD, const int* g
     double x[n];
 #pragma unroll
     for (int j = 0; j < n; ++j) x[j] = f[j * st];
-    fx_apply<n, n>(x, cD + k * (n * n), gD[k], FxRows{Dm, coef[k]}, [&](int a, double y) { f[a * st] = y; });
+    fx_apply<n, n, false>(x, cD + k * (n * n), gD[k], FxRows{Dm, coef[k]}, [&](int a, double y) { f[a * st] = y; });
   }
 }
 
@@ -184,7 +184,10 @@ __device__ __forceinline__ void time_fx(const double* F, double* q, const double
     }
     const double u0 = u[e];
     double* qv = q + v * NST + i;
-    fx_apply<n, n>(S, Kt, gK, FxRows{Ktd, 1.0}, [&](int m, double y) { qv[m * ND] = u0 - y; });
+    // (no look for steep lines: S itself is rounded at 2^-53 of the fluxes, which
+    // differ little between the time nodes, and lines of rounding noise, a uniform
+    // flow's, are as steep as a shock's)
+    fx_apply<n, n, true>(S, Kt, gK, FxRows{Ktd, 1.0}, [&](int m, double y) { qv[m * ND] = u0 - y; });
   }
 }
 
@@ -525,7 +528,7 @@ __device__ __forceinline__ void apply_pass_fx(const double* in, double* out, con
       double x[NI];
 #pragma unroll
       for (int j = 0; j < NI; ++j) x[j] = src[j * S];
-      fx_apply<NI, NO>(x, M.x, M.g, FxRows{M.d, 1.0}, [&](int a, double y) { dst[a * S] = y; });
+      fx_apply<NI, NO, false>(x, M.x, M.g, FxRows{M.d, 1.0}, [&](int a, double y) { dst[a * S] = y; });
     }
   }
 }
@@ -755,7 +758,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
         for (int k = 1; k < D; ++k) S += F[(k * NV + v) * NST + i];
         const double u0 = u[e];
         double* qv = q + v * NST + i;
-        fx_apply<1, n>(&S, kapx, gK, FxSums<n>{o->Kt}, [&](int m, double y) { qv[m * ND] = u0 - y; });
+        fx_apply<1, n, true>(&S, kapx, gK, FxSums<n>{o->Kt}, [&](int m, double y) { qv[m * ND] = u0 - y; });
       }
       it0 = 1;
     }
@@ -837,7 +840,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
         double x[n];
 #pragma unroll
         for (int m = 0; m < n; ++m) x[m] = F[kv * NST + i + m * ND];
-        fx_apply<n, 1>(x, wx, gw, FxRows{w, 1.0}, [&](int, double y) { fbar[e] = y; });
+        fx_apply<n, 1, true>(x, wx, gw, FxRows{w, 1.0}, [&](int, double y) { fbar[e] = y; });
       }
       __syncthreads();
     }
@@ -850,7 +853,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
       double x[n];
 #pragma unroll
       for (int j = 0; j < n; ++j) x[j] = f[j * st];
-      fx_apply<n, n>(x, cM + k * (n * n), gM[k], FxRows{o->Mvol, p.b.coef[k]}, [&](int a, double y) { f[a * st] = y; });
+      fx_apply<n, n, false>(x, cM + k * (n * n), gM[k], FxRows{o->Mvol, p.b.coef[k]}, [&](int a, double y) { f[a * st] = y; });
     }
     // space-time traces on the faces, trace[cell][k][side][v][ts + NF * m], by
     // lines: the n nodes of a line along axis k give both faces normal to k, and
@@ -864,7 +867,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
 #pragma unroll
         for (int j = 0; j < n; ++j) x[j] = f[j * st];
         double* t = tr + (2 * k) * (NV * NT) + vr;
-        fx_apply<n, 2>(x, phx, gph, FxRows{ph0, 1.0}, [&](int side, double y) { t[side * (NV * NT)] = y; });
+        fx_apply<n, 2, false>(x, phx, gph, FxRows{ph0, 1.0}, [&](int side, double y) { t[side * (NV * NT)] = y; });
       }
     __syncthreads();
     double* Uo = p.b.U[1 - p.cur] + cell * (NV * ND);

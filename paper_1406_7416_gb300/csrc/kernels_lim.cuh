@@ -1794,8 +1794,8 @@ __global__ void __launch_bounds__(128) k_lim_flux_d(Batch bt, int pass) {
         const double* a = qL + v * NST3;
         const double* b = qR + v * NST3;
         const double xa[3] = {a[0], a[stk], a[2 * stk]}, xb[3] = {b[0], b[stk], b[2 * stk]};
-        fx_apply<3, 1>(xa, ph[0], g, FxRows{o->phi13, 1.0}, [&](int, double y) { QL[v] = y; });
-        fx_apply<3, 1>(xb, ph[1], g, FxRows{o->phi03, 1.0}, [&](int, double y) { QR[v] = y; });
+        fx_apply<3, 1, true>(xa, ph[0], g, FxRows{o->phi13, 1.0}, [&](int, double y) { QL[v] = y; });
+        fx_apply<3, 1, true>(xb, ph[1], g, FxRows{o->phi03, 1.0}, [&](int, double y) { QR[v] = y; });
       }
       if (wall < 0) {
 #pragma unroll

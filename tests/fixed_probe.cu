@@ -29,7 +29,7 @@ __global__ void products(const double* M, const double* x, long long lines, doub
     double v[n];
 #pragma unroll
     for (int j = 0; j < n; ++j) v[j] = x[l * n + j];
-    fx_apply<n, n>(v, m, g, FxRows{M, 1.0}, [&](int a, double y) { out[l * n + a] = y; });
+    fx_apply<n, n, false>(v, m, g, FxRows{M, 1.0}, [&](int a, double y) { out[l * n + a] = y; });
   }
 }
 

@@ -114,3 +114,33 @@ def test_lines_with_a_nan_or_an_infinity(products, n, bad):
     x[2, n // 2] = bad
     y = products(np.full((n, n), 1.5), x)
     assert not np.isfinite(y[2]).any() and np.isfinite(np.delete(y, 2, axis=0)).all()
+
+
+def _operators(n):
+    from oracle.subcell import projection_matrix
+    b = Basis(n - 1)
+    P = projection_matrix(b, 2 * n - 1)
+    ops = {"D": b.D, "Mvol": b.w[None, :] * b.D.T / b.w[:, None]}
+    if n > 2:                               # (P of two nodes is not formed by these products)
+        ops.update(P_low=P[:n], P_mid=P[n // 2:n // 2 + n])
+    return ops
+
+
+@pytest.mark.parametrize("k", [7, 20, 40])
+@pytest.mark.parametrize("n", range(2, 11))
+def test_steep_lines(products, n, k):
+    """Lines with a spike at each node, and with a jump between each two, of 2^k: every row is as
+    accurate as an FMA chain, whose n roundings are each below 2^-53 of the sum of the terms'
+    magnitudes, a row that gives the large side little or no weight among them."""
+    rng = np.random.default_rng(n + k)
+    shapes = [np.arange(n) == j for j in range(n)] + [np.arange(n) < j for j in range(1, n)] + \
+        [np.arange(n) >= j for j in range(1, n)]
+    x = np.array([np.where(s, 2.0 ** k, 1.0) for s in shapes] * 4)
+    x *= rng.uniform(1, 1.9, x.shape) * rng.choice([-1, 1], x.shape)
+    for name, M in _operators(n).items():
+        y = products(M, x)
+        for l, row in enumerate(_exact(M, x)):
+            for a, v in enumerate(row):
+                mags = sum(abs(Fraction(float(m)) * Fraction(float(t))) for m, t in zip(M[a], x[l]))
+                err = abs(Fraction(float(y[l, a])) - v)
+                assert err <= n * mags / 2 ** 53, (name, l, a, float(err / mags) * 2 ** 53)
