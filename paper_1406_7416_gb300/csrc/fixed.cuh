@@ -215,7 +215,10 @@ __device__ __forceinline__ void fx_apply(const double* x, const FxOp* __restrict
     unsigned any = key;                                 // (a line of zeros, a flow at rest, has no sums)
 #pragma unroll
     for (int j = 0; j < n; ++j) any |= (unsigned)__double2loint(x[j]);
-    double v[n], y[ROWS];
+    // (in place where there are more results than elements: the projection's
+    // kernels then keep their registers, the predictor's do not)
+    double y[ROWS], w[n];
+    double* v = ROWS > n ? y : w;
 #pragma unroll
     for (int j = 0; j < n; ++j) v[j] = x[j];
     if (any) rows.template apply<n, ROWS>(v, y);
