@@ -361,6 +361,12 @@ __device__ __forceinline__ double widen_f32(float x) {
   return __hiloint2double((int)(s | (e11 << 20) | (m >> 3)), (int)(m << 29));
 }
 
+// The same for every float: subnormal ones (rare) by the conversion.
+__device__ __forceinline__ double widen_f32_any(float x) {
+  const unsigned u = __float_as_uint(x) * 2u;            // exponent and mantissa
+  return u != 0u && u < 0x01000000u ? (double)x : widen_f32(x);
+}
+
 // FP64 -> FP32 narrowing toward zero: the top 23 mantissa bits; magnitudes
 // below the FP32 normal range give zeros of their sign, above it the largest
 // finite float; infinities stay, NaNs stay NaN.

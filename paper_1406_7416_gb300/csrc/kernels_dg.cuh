@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(PredShape<D, N, MIXED>::bound, PredShape<D, N,
         __syncthreads();
       }
       if (!last64)
-        for (int e = tid; e < NV * NST; e += nth) q[e] = widen_f32(qf[e]);
+        for (int e = tid; e < NV * NST; e += nth) q[e] = widen_f32_any(qf[e]);
       it0 = n32;
     } else {
       // the first sweep starts from u (x) 1, whose fluxes and derivatives S are

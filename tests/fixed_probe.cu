@@ -1,4 +1,5 @@
-// Test probe: fx_apply of csrc/fixed.cuh on lines and operators from the host.
+// Test probe: fx_apply of csrc/fixed.cuh on lines and operators from the host, and
+// the widening of floats.
 #include <cuda_runtime.h>
 
 #include "../paper_1406_7416_gb300/csrc/fixed.cuh"
@@ -50,7 +51,23 @@ int run(int want, const double* M, const double* x, long long lines, double* out
   return e == cudaSuccess ? 0 : -3;
 }
 
+__global__ void widened(const float* x, int count, double* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < count) out[i] = widen_f32_any(x[i]);
+}
+
 }  // namespace
+
+extern "C" int widen_floats(const float* x, int count, double* out) {
+  double* d = nullptr;
+  if (cudaMalloc(&d, (sizeof(double) + sizeof(float)) * count) != cudaSuccess) return -2;
+  float* dx = reinterpret_cast<float*>(d + count);
+  cudaMemcpy(dx, x, sizeof(float) * count, cudaMemcpyHostToDevice);
+  widened<<<(count + 255) / 256, 256>>>(dx, count, d);
+  const cudaError_t e = cudaMemcpy(out, d, sizeof(double) * count, cudaMemcpyDeviceToHost);
+  cudaFree(d);
+  return e == cudaSuccess ? 0 : -3;
+}
 
 extern "C" int fixed_products(int n, const double* M, const double* x, long long lines, double* out) {
   return run<1>(n, M, x, lines, out);

@@ -16,18 +16,22 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture(scope="module")
-def products(tmp_path_factory):
+def probe(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("probe") / "fixed_probe.so")
     src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "fixed_probe.cu")
     subprocess.run([build_lib._nvcc()] + build_lib.NVCC_FLAGS + ["-shared", src, "-o", so], check=True)
-    lib = ctypes.CDLL(so)
+    return ctypes.CDLL(so)
+
+
+@pytest.fixture(scope="module")
+def products(probe):
     ptr = np.ctypeslib.ndpointer(np.float64, flags="C")
-    lib.fixed_products.argtypes = [ctypes.c_int, ptr, ptr, ctypes.c_longlong, ptr]
+    probe.fixed_products.argtypes = [ctypes.c_int, ptr, ptr, ctypes.c_longlong, ptr]
 
     def call(M, x):
         M, x = np.ascontiguousarray(M, float), np.ascontiguousarray(x, float)
         out = np.empty_like(x)
-        assert lib.fixed_products(M.shape[0], M, x, x.shape[0], out) == 0
+        assert probe.fixed_products(M.shape[0], M, x, x.shape[0], out) == 0
         return out
     return call
 
@@ -144,3 +148,17 @@ def test_steep_lines(products, n, k):
                 mags = sum(abs(Fraction(float(m)) * Fraction(float(t))) for m, t in zip(M[a], x[l]))
                 err = abs(Fraction(float(y[l, a])) - v)
                 assert err <= n * mags / 2 ** 53, (name, l, a, float(err / mags) * 2 ** 53)
+
+
+def test_widened_floats_are_exact(probe):
+    """FP32 results of the predictor's sweeps that an FP64 sweep goes on from: every float as its
+    double, subnormal ones, signed zeros and infinities included."""
+    rng = np.random.default_rng(1)
+    bits = np.concatenate([rng.integers(0, 2 ** 32, 20000), rng.integers(0, 2 ** 23, 2000),
+                           2 ** 31 + rng.integers(0, 2 ** 23, 2000),
+                           [0, 1, 2 ** 31, 2 ** 31 + 1, 2 ** 23 - 1, 2 ** 23, 0x7f800000, 0xff800000]])
+    x = bits.astype(np.uint32).view(np.float32)
+    x = x[~np.isnan(x)]
+    out = np.empty(x.size)
+    assert probe.widen_floats(x.ctypes.data_as(ctypes.c_void_p), x.size, out.ctypes.data_as(ctypes.c_void_p)) == 0
+    np.testing.assert_array_equal(out.view(np.uint64), x.astype(np.float64).view(np.uint64))
