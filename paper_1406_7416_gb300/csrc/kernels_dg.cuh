@@ -36,8 +36,7 @@ struct Dims {
 // threads capped at 102 registers, five blocks per SM (measured against four
 // blocks at N = 4 and 5: 8% and 4% faster; 160 threads: 17% slower at N = 4;
 // 256 threads: 40% slower), the 3D mixed kernel 160 threads, four blocks per
-// SM (9% faster than 128 at N = 3).  The FP64 kernel keeps the FP64 pipe busy
-// as it is and runs faster without the register cap.
+// SM (9% faster than 128 at N = 3).
 template <int D, int N, bool MIXED>
 struct PredShape {
   static constexpr bool wide = MIXED && D == 2 && N >= 6;
@@ -47,10 +46,16 @@ struct PredShape {
   // registers: <= 102 for the narrow mixed kernels (five 128- or four
   // 160-thread blocks per SM), <= 128 for the wide ones (two 256-thread or four
   // 128-thread blocks); <= 64 in FP64 up to N = 5, where the phases' barriers
-  // want more blocks beside each other (256^2 N = 5: 6.72 ms per step at 96
-  // registers, 6.37 at 80, 5.97 at 64, 6.12 at 48); no cap above (no difference)
+  // want more blocks beside each other; no cap above (no difference).  Measured
+  // (GB300, us per launch, FP64, the better block width, at most 64 / 80 / 128
+  // registers): 200^2 N = 1 191 / 191 / 180, N = 2 441 / 460 / 531, N = 3 807 /
+  // 819 / 904, N = 4 1958 / 2019 / 2240, N = 5 3899 / 4076 / 4523; 24^3 N = 1 117 /
+  // 118 / 126, N = 2 494 / 513 / 562, N = 3 1784 / 1834 / 1829.  The short phases
+  // of 2D N = 1 want the registers.
   static constexpr int min_blocks =
-      narrow3 ? 4 : ((MIXED && !wide) ? 5 : (MIXED ? 2 : ((D == 2 && N >= 6) ? 1 : 4)));
+      narrow3 ? 4
+              : ((MIXED && !wide) ? 5
+                                  : (MIXED ? 2 : ((D == 2 && N >= 6) ? 1 : (D == 2 && N == 1 ? 2 : 4))));
 };
 
 // ---------------------------------------------------------------------------

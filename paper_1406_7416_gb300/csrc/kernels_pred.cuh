@@ -565,8 +565,10 @@ template <int N>
 struct NodeLayout {
   using DM = Dims<2, N>;
   static constexpr int n = DM::n, ND = DM::ND, NST = DM::NST;
-  // cells per block: W n^2 nodes fill the block's warps (94% to 100%)
-  static constexpr int W = N == 5 ? 5 : (N == 4 ? 5 : (N == 3 ? 8 : (N == 2 ? 14 : 32)));
+  // cells per block: W n^2 nodes fill the block's warps (94% to 100%).  Measured
+  // (GB300, us per launch at 512^2): N = 1 32 cells 175, 16 cells 167; N = 2 14 416,
+  // 7 397; N = 3 8 834, 6 829; N = 4 5 1634, 4 1888
+  static constexpr int W = N == 5 ? 5 : (N == 4 ? 5 : (N == 3 ? 8 : (N == 2 ? 7 : 16)));
   static constexpr int threads = (W * ND + 31) / 32 * 32;
   static constexpr int blocks = 65536 / (threads * 80);     // at 80 registers
   // per cell: u (FP64 [4][ND]), then the fluxes (FP32 [2][4][NST]); after the
