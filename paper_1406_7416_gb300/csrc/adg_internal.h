@@ -39,16 +39,12 @@ struct Ops {
   double cq_phi[MAXNS * (MAXN + 1) * MAXN];   // phi_a(cq_x[p]) at [p*n+a]
   // degree-2 subcell basis (3 GL nodes)
   double w3[3], xi3[3], D3[9], Kt3[9], phi03[3], phi13[3];
-  // WENO3: coefficient matrices C[k][p*3+r] (stencil k, monomial p, cell r),
-  // nodal evaluation E[j*3+p] = xi3_j^p
-  double C[3][9];
-  double E[9];
   // float copies for the reduced-precision Picard sweeps
   float Df[MAXN * MAXN], Ktf[MAXN * MAXN];
   float wf[MAXN];             // time weights in FP32 (the split face fluxes)
-  // FP32 WENO3 (mixed precision): per stencil k the rows of C for c1, c2
-  // (Cf[k][0..2], Cf[k][3..5]) and the nodal values straight from the stencil
-  // averages, Wf[k][node * 3 + r] = sum_p E[node][p] C[k][p][r]
+  // FP32 WENO3 (mixed precision): per stencil k the coefficients of xi and xi^2
+  // from the stencil's three averages (Cf[k][0..2], Cf[k][3..5]) and the nodal
+  // values straight from them, Wf[k][node * 3 + r]
   float Cf[3][6];
   float Wf[3][9];
   // P1 for the integer pipes (fixed.cuh), with its scale exponent

@@ -6,17 +6,17 @@
 // A line of doubles is written as integers on the common scale of its largest
 // magnitude (59 bits and a sign, so 6 bits more than a double's 53 stay below
 // the largest element's last place), the operator's rows as 62-bit integers on
-// the scale of the largest row sum; the products accumulate in 128 bits of
-// which the low 64 are cut, and the result is rounded to a double once.
+// the scale of the largest row sum; the products of the high words with both
+// accumulate exactly, the low 64 bits of the sum are cut, and the result is
+// rounded to a double once.  Lines for which that scale does not do, steep ones
+// and those near the ends of the FP64 range, take the FP64 pipe (fx_apply).
 //
-// Measured (GB300, random operators and lines whose elements differ by up to
-// 2^70, against 113-bit arithmetic): relative 2-norm error 4.8e-17 at every n
-// of 3..10, the FMA chain 6.5e-17 (n = 4) to 1.1e-16 (n = 10).  Rate of whole
-// n x n products from and to doubles: 3.9e11 outputs/s at n = 3, 2.8e11 at
-// n = 6, 2.0e11 at n = 10, the FMA chain 1.9e11, 9.6e10 and 5.9e10 (its bound,
-// 2 FMA per clock): the integer form costs 0.45 + 0.1 n clocks of a
-// multiprocessor per 32 outputs, the FMA chain 0.5 n, and the FP64 pipe is
-// left to the non-linear work (fluxes).
+// Largest error of the derivative's rows on lines whose elements differ by
+// 2^4 and more, in units of the largest row sum times the line's largest element
+// (tests/test_gpu_fixed_products.py prints it; the FMA chain on the same lines):
+// n = 2 8.2e-17 (9.8e-17), n = 3 7.8e-17 (9.6e-17), n = 4 6.8e-17 (1.5e-16), n = 6
+// 4.1e-17 (1.1e-16), n = 8 4.2e-17 (1.4e-16), n = 10 2.9e-17 (9.1e-17).  What the
+// kernels gained stands at each of them.
 #pragma once
 
 #include <stdint.h>

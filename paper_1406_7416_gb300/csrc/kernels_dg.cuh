@@ -610,7 +610,8 @@ __device__ __forceinline__ int trace_index(int e, int& base, int& stk, int& s) {
 template <int D, int N, bool MIXED>
 __host__ __device__ constexpr size_t predictor_smem_bytes() {
   using DM = Dims<D, N>;
-  // u, q, F, fbar, the operators of PredOps and (split final stage) Mvol, w, phi
+  // u, q, F, fbar, the integer-pipe operators (cD, cM, Ktx, kapx, wx, phx of
+  // k_predictor), w and phi
   size_t d = (size_t)DM::NV * DM::ND + (size_t)DM::NV * DM::NST + (size_t)D * DM::NV * DM::NST +
              (size_t)D * DM::NV * DM::ND + (2 * D + 1) * DM::n * DM::n + 4 * DM::n + 3 * DM::n;
   // the FP32 sweep arrays qf, Ff live inside the FP64 flux array F (unused
@@ -1047,7 +1048,7 @@ struct FaceNode {
   const double *trL, *trR;   // (a missing side takes the other's)
 
   __device__ __forceinline__ FaceNode(const Params& p, int k, const int* at, int tsn) : ts(tsn) {
-    constexpr int n = DM::n, NV = DM::NV, NT = DM::NT;
+    constexpr int NV = DM::NV, NT = DM::NT;
     const Geo& g = p.geo;
     int L[3], R[3];
 #pragma unroll
@@ -1068,7 +1069,6 @@ struct FaceNode {
     trR = hasR ? p.b.trace + cell_index<D>(R, g) * csz + ((size_t)k * 2 + 0) * NV * NT : nullptr;
     if (!hasL) trL = trR;
     if (!hasR) trR = trL;
-    (void)n;
   }
   __device__ __forceinline__ bool inside() const { return hasL && hasR; }
 

@@ -1555,7 +1555,9 @@ __global__ void __launch_bounds__(256) k_lim_flux_t(Batch bt, int pass) {
 // T: the flux precision (double; float for the mixed-precision FP32 subcell
 // scheme, Rusanov only); the result is stored in FP64.
 // QT: the element type of the stored subcell predictor (float when it ran
-// wholly in FP32, see k_lim_predict).
+// wholly in FP32).  Launched as (float, float) without the register form of that
+// predictor, (float, double) with some of its sweeps in FP64, and (double, float)
+// with the Osher-type flux; (double, double) is k_lim_flux_d.
 template <int D, int N, int k, typename T, typename QT>
 __global__ void __launch_bounds__(256) k_lim_flux(Batch bt, int pass) {
   pass = lim_pass(bt, pass);
@@ -1616,8 +1618,6 @@ __global__ void __launch_bounds__(256) k_lim_flux(Batch bt, int pass) {
     const QT* qR = reinterpret_cast<const QT*>(p.b.qsub) + (jR * NED + sr) * NV * NST3;
     // a sub-face on a reflecting wall takes its flux between the interior
     // trace and its mirror image (no mass or energy through the wall)
-    // (the troubled-cell list is read only when the face can be a wall: the
-    // no-allocation entry point runs this kernel with periodic kinds and no list)
     int wall = 0;                          // -1: low wall (ghost left), +1: high wall (ghost right)
     const bool lo_wall = fc[k] == 0 && p.geo.bc[2 * k] == ADG_BC_REFLECTIVE;
     const bool hi_wall = fc[k] == Ns && p.geo.bc[2 * k + 1] == ADG_BC_REFLECTIVE;
@@ -1631,10 +1631,10 @@ __global__ void __launch_bounds__(256) k_lim_flux(Batch bt, int pass) {
     T acc[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) acc[v] = T(0);
-    const float gf = p.b.coef_f ? p.b.coef_f[7] : (float)p.gamma;
+    const float gf = p.b.coef_f[7];
     // tangential x time nodes: digits over axes != k, then time
     for (int t = 0; t < ND3; ++t) {
-      int base = 0, tt = t, wmul = 1;
+      int base = 0, tt = t;
       T wt = T(1);
       int st = 1;
 #pragma unroll
@@ -1650,7 +1650,6 @@ __global__ void __launch_bounds__(256) k_lim_flux(Batch bt, int pass) {
       const int m = tt;                 // remaining digit: time node
       wt *= m == 0 ? w3t[0] : (m == 1 ? w3t[1] : w3t[2]);
       base += m * ND3;
-      (void)wmul;
       T QL[NV], QR[NV], G[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
@@ -1780,7 +1779,9 @@ __global__ void __launch_bounds__(128) k_lim_flux_d(Batch bt, int pass) {
           jR = j2;
           sr -= across;
         }
-        // reflecting walls: as in k_lim_flux
+        // reflecting walls: as in k_lim_flux (the list of troubled cells is read
+        // only where the face can be a wall: the no-allocation entry point runs
+        // this kernel with periodic kinds, no list and no table of neighbours)
         const int side = fck == 0 ? 0 : 1;
         if (p.geo.bc[2 * k + side] == ADG_BC_REFLECTIVE) {
           const long long cell = p.b.list[1 - p.cur][pass * p.chunk + j];

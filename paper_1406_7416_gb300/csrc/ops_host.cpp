@@ -229,8 +229,6 @@ void build_ops(int N, Ops* o) {
       o->D3[i] = (double)D3[i];
       o->Kt3[i] = (double)K3[i];
     }
-    for (int j = 0; j < 3; ++j)
-      for (int p = 0; p < 3; ++p) o->E[j * 3 + p] = (double)powl(x3[j], (ld)p);
   }
   // WENO3 stencils {s-2..s}, {s-1..s+1}, {s..s+2}: A[r][p] = int_o^{o+1} xi^p
   for (int k = 0; k < 3; ++k) {
@@ -241,7 +239,6 @@ void build_ops(int N, Ops* o) {
       for (int p = 0; p < 3; ++p) A[r * 3 + p] = (powl(hi, (ld)(p + 1)) - powl(lo, (ld)(p + 1))) / (p + 1);
     }
     invert(A, 3);   // A^{-1}[p][r]: monomial p from cell r
-    for (int i = 0; i < 9; ++i) o->C[k][i] = (double)A[i];
     for (int r = 0; r < 3; ++r) {
       o->Cf[k][r] = (float)A[3 + r];
       o->Cf[k][3 + r] = (float)A[6 + r];
