@@ -164,12 +164,13 @@ struct FxSums {
   const double* m;
   template <int n, int ROWS>
   __device__ __forceinline__ void apply(const double* x, double* y) const {
+    const double x0 = x[0];                             // (y may lie over x)
 #pragma unroll 1
     for (int a = 0; a < ROWS; ++a) {
       double s = 0.0;
 #pragma unroll 1
       for (int j = 0; j < L; ++j) s += m[a * L + j];
-      y[a] = s * x[0];
+      y[a] = s * x0;
     }
   }
 };

@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(128) k_lim_patch(Batch bt, int pass) {
 // sigma_k + eps over the power of two of the smallest and a_k = lambda_k
 // prod_{j != k} t_j^8 they are a_k / sum a, one division.  t_k is cut at 2^50, so
 // that no product overflows whatever the data's magnitude, and a stencil that far
-// from the smoothest has no weight (below 2^-380 of the largest: what it would
+// from the smoothest has no weight (below 2^-370 of the largest: what it would
 // add lies under the last place of the smoothest one's differences).
 //
 // Measured (GB300, 3D explosion 33 x 29 x 30, N = 3): the three sweeps of 5611

@@ -34,10 +34,38 @@ __global__ void products(const double* M, const double* x, long long lines, doub
   }
 }
 
+// out[line][n] = (row sums of M) x[line][0], the predictor's first time solve
 template <int n>
-int run(int want, const double* M, const double* x, long long lines, double* out) {
+__global__ void sums(const double* M, const double* x, long long lines, double* out) {
+  __shared__ FxOp m[n];
+  __shared__ int g;
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int a = 0; a < n; ++a) {
+      double r = 0.0;
+      for (int j = 0; j < n; ++j) r += fabs(M[a * n + j]);
+      s = r > s ? r : s;
+    }
+    g = fx_scale(s);
+  }
+  __syncthreads();
+  for (int a = threadIdx.x; a < n; a += blockDim.x) {
+    double r = 0.0;
+    for (int j = 0; j < n; ++j) r += M[a * n + j];
+    m[a] = fx_op(r, g);
+  }
+  __syncthreads();
+  for (long long l = blockIdx.x * (long long)blockDim.x + threadIdx.x; l < lines;
+       l += (long long)gridDim.x * blockDim.x) {
+    const double v = x[l * n];
+    fx_apply<1, n, true>(&v, m, g, FxSums<n>{M}, [&](int a, double y) { out[l * n + a] = y; });
+  }
+}
+
+template <int n>
+int run(int want, bool sum, const double* M, const double* x, long long lines, double* out) {
   if (want != n) {
-    if constexpr (n < 10) return run<n + 1>(want, M, x, lines, out);
+    if constexpr (n < 10) return run<n + 1>(want, sum, M, x, lines, out);
     return -1;
   }
   double* d = nullptr;
@@ -45,7 +73,8 @@ int run(int want, const double* M, const double* x, long long lines, double* out
   double *dx = d + n * n, *dout = dx + lines * n;
   cudaMemcpy(d, M, sizeof(double) * n * n, cudaMemcpyHostToDevice);
   cudaMemcpy(dx, x, sizeof(double) * lines * n, cudaMemcpyHostToDevice);
-  products<n><<<64, 128>>>(d, dx, lines, dout);
+  if (sum) sums<n><<<64, 128>>>(d, dx, lines, dout);
+  else products<n><<<64, 128>>>(d, dx, lines, dout);
   const cudaError_t e = cudaMemcpy(out, dout, sizeof(double) * lines * n, cudaMemcpyDeviceToHost);
   cudaFree(d);
   return e == cudaSuccess ? 0 : -3;
@@ -70,5 +99,9 @@ extern "C" int widen_floats(const float* x, int count, double* out) {
 }
 
 extern "C" int fixed_products(int n, const double* M, const double* x, long long lines, double* out) {
-  return run<1>(n, M, x, lines, out);
+  return run<1>(n, false, M, x, lines, out);
+}
+
+extern "C" int fixed_sums(int n, const double* M, const double* x, long long lines, double* out) {
+  return run<1>(n, true, M, x, lines, out);
 }

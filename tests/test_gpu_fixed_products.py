@@ -111,6 +111,28 @@ def test_lines_at_the_ends_of_the_range(products, n, e):
             assert abs(Fraction(float(y[l, a])) - v) <= bar, (l, a)
 
 
+@pytest.mark.parametrize("n", range(1, 11))
+@pytest.mark.parametrize("e", [-1060, -1000, -958, 0, 974, 980, 1010])
+def test_row_sums_over_the_range(probe, n, e):
+    """The first time solve, each row's sum times one value: an operator entry and the result round."""
+    M = Basis(n - 1).Ktau if n > 1 else np.array([[1.7]])
+    rng = np.random.default_rng(n)
+    x = np.repeat(np.ldexp(rng.uniform(0.5, 1, (30, 1)) * rng.choice([-1, 1], (30, 1)), e), n, axis=1)
+    x[3] = 0.0
+    y = np.empty_like(x)
+    ptr = np.ctypeslib.ndpointer(np.float64, flags="C")
+    probe.fixed_sums.argtypes = [ctypes.c_int, ptr, ptr, ctypes.c_longlong, ptr]
+    assert probe.fixed_sums(n, np.ascontiguousarray(M), x, x.shape[0], y) == 0
+    sums = [sum(Fraction(float(v)) for v in row) for row in M]
+    scale = Fraction(float(np.abs(M).sum(axis=1).max()))
+    for l in range(x.shape[0]):
+        for a in range(n):
+            v = sums[a] * Fraction(float(x[l, a]))
+            # the row's sum in doubles (n roundings), the product, and in integers 2^-55 of the scale
+            bar = (n + 4) * scale * abs(Fraction(float(x[l, a]))) / 2 ** 53 + Fraction(1, 2 ** 1074)
+            assert abs(Fraction(float(y[l, a])) - v) <= bar, (l, a)
+
+
 @pytest.mark.parametrize("n", [1, 2, 5])
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
 def test_lines_with_a_nan_or_an_infinity(products, n, bad):
