@@ -130,9 +130,9 @@ __device__ __forceinline__ void picard_time(T* __restrict__ q, const UT* __restr
 // the axes; the phases run by lines, each line read and converted once for its
 // n outputs, and the derivative phase works in place, so that the axes need no
 // barrier between them.  Measured (GB300, predictor phase per step): 256^2
-// N = 5 FP64 17.1 -> 6.7 ms, 67 x 53 N = 6 FP64 1.93 -> 0.73 ms, 33 x 29 x 30
-// N = 3 FP64 7.75 -> 3.19 ms, 200^2 N = 9 mixed (nine FP32 sweeps and this one)
-// 17.0 -> 11.1 ms.
+// N = 5 FP64 17.1 -> 6.4 ms, 67 x 53 N = 6 FP64 1.93 -> 0.77 ms, 33 x 29 x 30
+// N = 3 FP64 7.75 -> 3.68 ms, 200^2 N = 9 mixed (nine FP32 sweeps and this one)
+// 17.0 -> 11.4 ms.
 //
 // Fluxes of `nodes` space-time nodes (all NST, or the ND of time node 0).
 template <int D, int n>
@@ -448,7 +448,7 @@ __device__ __forceinline__ void apply_pass_ct(const T* __restrict__ in, T* __res
 // averages itself (no copy of them in shared memory, one barrier fewer) and
 // reduces its extremes by warp_max_key: 5022 -> 3774 instructions per 2D N = 5
 // cell.  Measured (GB300), corrector and detector per step, mixed: 512^2 N = 5
-// 2.14 -> 1.86 ms, 200^2 N = 9 1.65 -> 1.35, 64^3 N = 3 10.1 -> 8.1.
+// 2.14 -> 1.91 ms, 200^2 N = 9 1.65 -> 1.32, 64^3 N = 3 10.1 -> 8.4.
 template <int D, int N, int K>
 __device__ __forceinline__ void project_pass_f(const float* in, float* out, int tid, int nth) {
   constexpr int NV = D + 2, NI = N + 1, NO = 2 * N + 1;

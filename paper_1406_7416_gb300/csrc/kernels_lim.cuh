@@ -729,10 +729,10 @@ __device__ __noinline__ void sub_predict_fp64(double* x, const double* ck, doubl
 // q_m = u - kappa_m S with kappa = Ktau 1.  FP64 operations per sweep, node and
 // variable: the flux (4.4 in 3D, 4.1 in 2D) and one subtraction.
 //
-// Measured (GB300, 3D explosion 33 x 29 x 30, N = 3): 56 ms for 5611 troubled
-// cells (3.6 million subcells; FP64 pipe 72% busy, 208 FP64 instructions per
-// subcell), the former kernel with FP64 contractions from shared memory 174 ms
-// for 4883 (mean of two launches); 2D N = 5, 146 patches: 351 -> 100 us.
+// Measured (GB300, 3D explosion 33 x 29 x 30, N = 3): 47 ms for 4883 troubled
+// cells (mean of two launches; 3.1 million subcells, FP64 pipe 63% busy), the
+// former kernel with FP64 contractions from shared memory 174 ms; 2D N = 5, 146
+// patches: 351 -> 113 us.
 template <int D, int N, typename WT>
 __global__ void __launch_bounds__(128) k_lim_predict_i(Batch bt) {
   using DM = Dims<D, N>;
